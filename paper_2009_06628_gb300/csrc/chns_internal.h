@@ -25,6 +25,7 @@ struct DevMesh {
 };
 
 struct SolverWS;  // Newton-Krylov workspace (solver.cu)
+struct PrecondWS; // preconditioner operators and vectors (precond.cu)
 struct MGHier;    // geometric multigrid hierarchy of the pressure Schur Laplacian (multigrid.cu)
 
 struct chns_mesh {
@@ -56,6 +57,7 @@ struct chns_mesh {
     unsigned int* d_flags = nullptr; // bit 0: a tau radicand was not positive
     SolverWS* ws = nullptr;
     MGHier* mg = nullptr;
+    PrecondWS* pre = nullptr;        // assembled operators of the preconditioners (precond.cu)
     // scatter strategy of the element kernels (0 atomics, 1 colouring, 2 warp-aggregated)
     int32_t scatter = 0;
     int32_t* d_elist = nullptr;          // elements sorted by colour (Morton order within one)
@@ -132,7 +134,7 @@ cudaError_t transfer_apply_f32(const TransferDev& T, bool transpose, bool add, c
                                cudaStream_t s);
 
 // Geometric multigrid hierarchy of the pressure Schur Laplacian (multigrid.cu builds it,
-// solver.cu sets it up and applies V-cycles).  Level 0 is the mesh itself; level l + 1 caps
+// precond.cu assembles its levels and applies V-cycles).  Level 0 is the mesh itself; level l + 1 caps
 // every leaf of level l at (deepest level of l) - 1, which keeps the octree complete and
 // 2:1 balanced and makes its Q1 space a subspace of level l's.
 struct MGLevel {
@@ -141,23 +143,10 @@ struct MGLevel {
     int64_t N = 0, E = 0;
     TransferDev P;              // this level -> level - 1 (level >= 1)
     int32_t* fmap = nullptr;    // for every element of level - 1: its element on this level
-    float* ce = nullptr;        // element coefficients of the Schur Laplacian
-    float* dinv = nullptr;      // inverse diagonal
-    float* bnd = nullptr;       // absolute-row-sum bounds (Gershgorin)
-    float* b = nullptr;         // right-hand side, solution, residual
-    float* x = nullptr;
-    float* t = nullptr;
-    float* cr = nullptr;        // Chebyshev work vectors
-    float* cx = nullptr;
-    float* cd = nullptr;
-    float* cy = nullptr;
-    std::vector<float> c1, c2;  // Chebyshev recurrence coefficients of this level
-    float inv_theta = 0.0f;
-    int deg = 0;
+    float* ce = nullptr;        // element coefficients of the Schur Laplacian (level >= 1)
 };
 struct MGHier {
     std::vector<MGLevel> lv;
-    unsigned int* kmax = nullptr;   // per-level Gershgorin bounds (float bits)
 };
 chns_status mg_hier_build(chns_mesh* m);   // no-op when m->mg exists
 void chns_mg_free(MGHier* mg);

@@ -312,9 +312,11 @@ extern "C" chns_status chns_mesh_create(int32_t dim, int32_t max_level, int64_t 
 
 void chns_solver_ws_free(SolverWS* ws);  // solver.cu
 void chns_mg_free(MGHier* mg);           // multigrid.cu
+void precond_free(PrecondWS* p);         // precond.cu
 
 extern "C" void chns_mesh_destroy(chns_mesh* m) {
     if (!m) return;
+    precond_free(m->pre);
     if (m->ws) chns_solver_ws_free(m->ws);
     if (m->mg) chns_mg_free(m->mg);
     cudaFree(m->d_e2n);

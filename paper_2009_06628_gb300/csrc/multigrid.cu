@@ -267,15 +267,6 @@ extern "C" chns_status chns_coarsen_leaves(int32_t dim, int32_t max_level, int64
     return CHNS_OK;
 }
 
-static chns_status alloc_level(MGLevel& L) {
-    cudaError_t e = cudaSuccess;
-    for (float** p : {&L.dinv, &L.bnd, &L.b, &L.x, &L.t, &L.cr, &L.cx, &L.cd, &L.cy})
-        if (e == cudaSuccess) e = cudaMalloc((void**)p, (size_t)std::max<int64_t>(L.N, 1) * sizeof(float));
-    // level 0 reads the Schur coefficients of the solver workspace; coarse levels own theirs
-    if (e == cudaSuccess && L.mesh) e = cudaMalloc((void**)&L.ce, (size_t)std::max<int64_t>(L.E, 1) * sizeof(float));
-    return e == cudaSuccess ? CHNS_OK : chns_cuda_status(e, "cudaMalloc(multigrid level)");
-}
-
 chns_status mg_hier_build(chns_mesh* m) {
     if (m->mg) return CHNS_OK;
     MGHier* mg = new MGHier();
@@ -313,11 +304,11 @@ chns_status mg_hier_build(chns_mesh* m) {
         mg->lv.push_back(L);
         cur = cm;
     }
-    if (st == CHNS_OK)
-        for (size_t l = 0; l < mg->lv.size() && st == CHNS_OK; ++l) st = alloc_level(mg->lv[l]);
-    if (st == CHNS_OK) {
-        cudaError_t e = cudaMalloc((void**)&mg->kmax, 64 * sizeof(unsigned int));
-        if (e != cudaSuccess) st = chns_cuda_status(e, "cudaMalloc(multigrid bounds)");
+    for (MGLevel& L : mg->lv) {
+        // level 0 reads the coefficients of the solver workspace
+        if (st != CHNS_OK || !L.mesh) continue;
+        const cudaError_t e = cudaMalloc((void**)&L.ce, (size_t)std::max<int64_t>(L.E, 1) * sizeof(float));
+        if (e != cudaSuccess) st = chns_cuda_status(e, "cudaMalloc(multigrid level)");
     }
     if (st != CHNS_OK) {
         chns_mg_free(mg);
@@ -332,10 +323,9 @@ void chns_mg_free(MGHier* mg) {
     for (auto& L : mg->lv) {
         transfer_free(&L.P);
         cudaFree(L.fmap);
-        for (float* p : {L.ce, L.dinv, L.bnd, L.b, L.x, L.t, L.cr, L.cx, L.cd, L.cy}) cudaFree(p);
+        cudaFree(L.ce);
         if (L.mesh) chns_mesh_destroy(L.mesh);
     }
-    cudaFree(mg->kmax);
     delete mg;
 }
 

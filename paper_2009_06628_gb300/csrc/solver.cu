@@ -22,6 +22,7 @@
 
 #include "chns_internal.h"
 #include "pointwise.cuh"
+#include "precond.h"
 #include "reduce.cuh"
 
 struct SolverWS {
@@ -49,51 +50,18 @@ struct SolverWS {
     double* hsc = nullptr;   // pinned host scalars
     cudaEvent_t ev[16] = {};  // J x, preconditioner build / apply and Gram-Schmidt timing (two sets
                               // of J x / apply events alternate between Arnoldi steps)
-    // pressure Schur-complement approximation (FP32)
-    float* ce = nullptr;     // E element coefficients
-    float* kdinv = nullptr;  // N inverse diagonal
-    // CUDA graphs of the pressure Schur apply (2 + 2 (degree - 1) launches), captured on
-    // a private stream per (input, output, output type) and Chebyshev set-up
-    struct SchurGraph {
-        cudaGraphExec_t exec = nullptr;
-        const void* vin = nullptr;
-        void* zout = nullptr;
-        size_t to = 0;
-        int gen = -1;
-        int nk = 0;   // kernels in the graph (launch accounting)
-    } sgraph[4];
-    cudaStream_t cap = nullptr;
-    int schur_gen = 0;
+    float* ce = nullptr;     // E element coefficients of the pressure Schur approximation
+    cudaStream_t cap = nullptr;   // capture stream of the Gram-Schmidt graphs
     bool no_graphs = false;
     // CUDA graphs of the Gram-Schmidt sequence of Arnoldi step j (its kernels take k = j + 1
     // and fixed workspace pointers), captured at first use
     cudaGraphExec_t orth_exec[257] = {};
-    float* kbnd = nullptr;   // N bounds of the absolute row sums of the Schur Laplacian
-    unsigned int* kmax = nullptr;  // max_p kbnd[p] / diag[p] (float bits)
-    float* cr = nullptr;     // N Chebyshev work vectors
-    float* cx = nullptr;
-    float* cd = nullptr;
-    float* cy = nullptr;
     double* part = nullptr;  // per-block partials of the fused orthogonalisation reductions
-    // Cahn-Hilliard block (pc_type 2), FP32 nodal work arrays
-    float* ch_dinv = nullptr;  // inverse diagonal of M + eps K
-    float* ch_ml = nullptr;    // lumped mass (node integrals)
-    float* ch_psi2 = nullptr;  // psi''(phi~) at the nodes
-    float* ch_a = nullptr;
-    float* ch_b = nullptr;
-    float* ch_c = nullptr;
-    float* ch_rm = nullptr;
-    std::vector<float> ch_c1, ch_c2;
-    float ch_inv_theta = 0.0f, ch_eps = 0.0f;
-    std::vector<float> cheb_c1, cheb_c2;
-    float cheb_inv_theta = 0.0f;
-    int kref_dim = 0;
+    float* ch_psi2 = nullptr;  // psi''(phi~) at the nodes (Cahn-Hilliard block)
 };
 
 void chns_solver_ws_free(SolverWS* ws) {
     if (!ws) return;
-    for (auto& g : ws->sgraph)
-        if (g.exec) cudaGraphExecDestroy(g.exec);
     for (auto& g : ws->orth_exec)
         if (g) cudaGraphExecDestroy(g);
     if (ws->cap) cudaStreamDestroy(ws->cap);
@@ -117,21 +85,8 @@ void chns_solver_ws_free(SolverWS* ws) {
     cudaFree(ws->Pinv64);
     cudaFree(ws->sc);
     cudaFree(ws->ce);
-    cudaFree(ws->kdinv);
-    cudaFree(ws->kbnd);
-    cudaFree(ws->kmax);
-    cudaFree(ws->cr);
-    cudaFree(ws->cx);
-    cudaFree(ws->cd);
-    cudaFree(ws->cy);
     cudaFree(ws->part);
-    cudaFree(ws->ch_dinv);
-    cudaFree(ws->ch_ml);
     cudaFree(ws->ch_psi2);
-    cudaFree(ws->ch_a);
-    cudaFree(ws->ch_b);
-    cudaFree(ws->ch_c);
-    cudaFree(ws->ch_rm);
     if (ws->hsc) cudaFreeHost(ws->hsc);
     for (auto& e : ws->ev)
         if (e) cudaEventDestroy(e);
@@ -146,7 +101,10 @@ constexpr int ORTH_MAX_BX = 1024;   // row blocks of the fused orthogonalisation
 chns_status ensure_ws(chns_mesh* m, int restart) {
     SolverWS* ws = m->ws;
     if (ws && ws->restart >= restart) return CHNS_OK;
-    if (ws) chns_solver_ws_free(ws);
+    if (ws) {
+        precond_drop_graphs(m);   // they hold the old workspace's vectors
+        chns_solver_ws_free(ws);
+    }
     m->ws = nullptr;
     ws = new SolverWS();
     ws->restart = restart;
@@ -177,16 +135,8 @@ chns_status ensure_ws(chns_mesh* m, int restart) {
     A((void**)&ws->Pinv64, nb * sizeof(double));
     A((void**)&ws->sc, MAXSC * sizeof(double));
     A((void**)&ws->ce, (size_t)m->dm.E * sizeof(float));
-    A((void**)&ws->kdinv, (size_t)m->dm.N * sizeof(float));
-    A((void**)&ws->kbnd, (size_t)m->dm.N * sizeof(float));
-    A((void**)&ws->kmax, sizeof(unsigned int));
-    A((void**)&ws->cr, (size_t)m->dm.N * sizeof(float));
-    A((void**)&ws->cx, (size_t)m->dm.N * sizeof(float));
-    A((void**)&ws->cd, (size_t)m->dm.N * sizeof(float));
-    A((void**)&ws->cy, (size_t)m->dm.N * sizeof(float));
     A((void**)&ws->part, (size_t)ORTH_MAX_BX * (MAXSC / 32 + 1) * 9 * sizeof(double));
-    for (float** p : {&ws->ch_dinv, &ws->ch_ml, &ws->ch_psi2, &ws->ch_a, &ws->ch_b, &ws->ch_c, &ws->ch_rm})
-        A((void**)p, (size_t)m->dm.N * sizeof(float));
+    A((void**)&ws->ch_psi2, (size_t)m->dm.N * sizeof(float));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&ws->hsc, MAXSC * sizeof(double));
     for (auto& ev : ws->ev)
         if (e == cudaSuccess) e = cudaEventCreate(&ev);
@@ -816,547 +766,28 @@ cudaError_t pc_build_launch(const chns_mesh* m, const PhysConst& pc, const T* Uo
     return cudaGetLastError();
 }
 
-// ---------------- pressure Schur-complement approximation ----------------
-// Eliminating v^{k+1} from the momentum rows (dominated by rho M / dt at small dt)
-// leaves, for p^{k+1}, approximately the Laplacian (grad q, dt/(2 rho We) grad p)
-// (the Galerkin divergence and the stabilisation rows together).  Its inverse is
-// approximated by a Jacobi-preconditioned Chebyshev iteration of fixed degree (a
-// fixed polynomial, so GMRES sees a linear preconditioner).
-__constant__ float c_Kref[64];   // Q1 stiffness of the unit element (2-point Gauss)
-
-void kref_host(int D, float* K) {
-    const int NC = 1 << D;
-    const double gp = 0.78867513459481288225, gm = 0.21132486540518711775;
-    for (int a = 0; a < NC; ++a)
-        for (int b = 0; b < NC; ++b) {
-            double sum = 0.0;
-            for (int q = 0; q < NC; ++q)
-                for (int k = 0; k < D; ++k) {
-                    double da = ((a >> k) & 1) ? 1.0 : -1.0, db = ((b >> k) & 1) ? 1.0 : -1.0;
-                    for (int j = 0; j < D; ++j) {
-                        if (j == k) continue;
-                        da *= (((a >> j) & 1) == ((q >> j) & 1)) ? gp : gm;
-                        db *= (((b >> j) & 1) == ((q >> j) & 1)) ? gp : gm;
-                    }
-                    sum += da * db;
-                }
-            K[a * NC + b] = (float)(sum / (double)NC);   // |det J| = (1/2)^d, unit Gauss weights
-        }
-}
-
-template <int D>
-__device__ __forceinline__ void schur_corners(const DevMesh& m, int64_t e, int par[][4], int np[]) {
-    constexpr int NC = 1 << D;
-    for (int a = 0; a < NC; ++a) {
-        const int ent = m.e2n[e * NC + a];
-        if (ent >= 0) {
-            np[a] = 1;
-            par[a][0] = ent;
-        } else {
-            const int4 hp = reinterpret_cast<const int4*>(m.hang)[-ent - 1];
-            par[a][0] = hp.x;
-            par[a][1] = hp.y;
-            par[a][2] = hp.z;
-            par[a][3] = hp.w;
-            np[a] = hp.z < 0 ? 2 : 4;
-        }
-    }
-}
-
-// Diagonal of the Schur Laplacian (constraint cross terms within a corner's parents
-// are dropped: it only scales the Chebyshev iteration) and, per node p, a bound on the
-// absolute row sum of the constrained operator: sum_q |K_pq| <= sum over the corners a
-// that map to p of w_ap sum_b |K_e[a][b]| (the constraint weights of a corner sum to 1).
-template <int D>
-__global__ void schur_diag_kernel(DevMesh m, const float* __restrict__ ce, float* __restrict__ dg,
-                                  float* __restrict__ bnd) {
-    constexpr int NC = 1 << D;
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= m.E) return;
-    const float h = (float)ldexp(m.hi - m.lo, -(int)m.level[e]);
-    const float ch = ce[e] * (D == 2 ? 1.0f : h);
-    int par[NC][4], np[NC];
-    schur_corners<D>(m, e, par, np);
-    for (int a = 0; a < NC; ++a) {
-        const float w = np[a] == 1 ? 1.0f : (np[a] == 2 ? 0.5f : 0.25f);
-        float rs = 0.0f;
-        for (int b = 0; b < NC; ++b) rs += fabsf(c_Kref[a * NC + b]);
-        for (int j = 0; j < np[a]; ++j) {
-            atomicAdd(dg + par[a][j], w * w * ch * c_Kref[a * NC + a]);
-            atomicAdd(bnd + par[a][j], w * ch * rs);
-        }
-    }
-}
-
-// out = max_n bnd[n] dinv[n] (non-negative floats compare like their bit patterns)
-__global__ void gershgorin_max_kernel(const float* __restrict__ bnd, const float* __restrict__ dinv, int64_t N,
-                                      unsigned int* __restrict__ out) {
-    float v = 0.0f;
-    for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (int64_t)gridDim.x * blockDim.x)
-        v = fmaxf(v, bnd[n] * dinv[n]);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
-    if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(v));
-}
-
-// y += sgn K_c x  (y zeroed, or holding a right-hand side, by the caller)
-template <int D>
-__global__ void schur_matvec_kernel(DevMesh m, const float* __restrict__ ce, const float* __restrict__ x,
-                                    float* __restrict__ y, float sgn = 1.0f) {
-    constexpr int NC = 1 << D;
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= m.E) return;
-    const float h = (float)ldexp(m.hi - m.lo, -(int)m.level[e]);
-    const float ch = sgn * ce[e] * (D == 2 ? 1.0f : h);
-    int par[NC][4], np[NC];
-    schur_corners<D>(m, e, par, np);
-    float xl[NC];
-    for (int a = 0; a < NC; ++a) {
-        const float w = np[a] == 1 ? 1.0f : (np[a] == 2 ? 0.5f : 0.25f);
-        float s = 0.0f;
-        for (int j = 0; j < np[a]; ++j) s += w * __ldg(x + par[a][j]);
-        xl[a] = s;
-    }
-    for (int a = 0; a < NC; ++a) {
-        float s = 0.0f;
-#pragma unroll
-        for (int b = 0; b < NC; ++b) s += c_Kref[a * NC + b] * xl[b];
-        s *= ch;
-        const float w = np[a] == 1 ? 1.0f : (np[a] == 2 ? 0.5f : 0.25f);
-        for (int j = 0; j < np[a]; ++j) atomicAdd(y + par[a][j], w * s);
-    }
-}
-
-__global__ void axpbyf_kernel(float a, float* __restrict__ x, int64_t n) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) x[i] *= a;
-}
-__constant__ float c_Mref[64];   // Q1 consistent mass of the unit element (2-point Gauss)
-
-void mref_host(int D, float* Mr) {
-    const int NC = 1 << D;
-    const double gp = 0.78867513459481288225, gm = 0.21132486540518711775;
-    for (int a = 0; a < NC; ++a)
-        for (int b = 0; b < NC; ++b) {
-            double sum = 0.0;
-            for (int q = 0; q < NC; ++q) {
-                double na = 1.0, nb = 1.0;
-                for (int k = 0; k < D; ++k) {
-                    na *= (((a >> k) & 1) == ((q >> k) & 1)) ? gp : gm;
-                    nb *= (((b >> k) & 1) == ((q >> k) & 1)) ? gp : gm;
-                }
-                sum += na * nb;
-            }
-            Mr[a * NC + b] = (float)(sum / (double)NC);   // |det J| = (1/2)^d for h = 1
-        }
-}
-
-// y += (alpha M + beta K) x, or its diagonal (DIAG), on the Q1 space with constraints;
-// DIAG also accumulates into bnd the absolute-row-sum bounds used for the Gershgorin
-// top of the spectrum (as for the pressure Schur Laplacian)
-template <int D, bool DIAG>
-__global__ void mk_kernel(DevMesh m, float span, float alpha, float beta, const float* __restrict__ x,
-                          float* __restrict__ y, float* __restrict__ bnd = nullptr) {
-    constexpr int NC = 1 << D;
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= m.E) return;
-    const float h = ldexpf(span, -(int)m.level[e]);
-    const float hd2 = (D == 2) ? 1.0f : h;            // h^(d-2)
-    const float hd = hd2 * h * h;                      // h^d
-    const float am = alpha * hd, bk = beta * hd2;
-    int par[NC][4], np[NC];
-    schur_corners<D>(m, e, par, np);
-    if (DIAG) {
-        for (int a = 0; a < NC; ++a) {
-            const float w = np[a] == 1 ? 1.0f : (np[a] == 2 ? 0.5f : 0.25f);
-            const float v = am * c_Mref[a * NC + a] + bk * c_Kref[a * NC + a];
-            float rs = 0.0f;
-            for (int b = 0; b < NC; ++b) rs += fabsf(am * c_Mref[a * NC + b] + bk * c_Kref[a * NC + b]);
-            for (int j = 0; j < np[a]; ++j) {
-                atomicAdd(y + par[a][j], w * w * v);
-                if (bnd) atomicAdd(bnd + par[a][j], w * rs);
-            }
-        }
-        return;
-    }
-    float xl[NC];
-    for (int a = 0; a < NC; ++a) {
-        const float w = np[a] == 1 ? 1.0f : (np[a] == 2 ? 0.5f : 0.25f);
-        float sacc = 0.0f;
-        for (int j = 0; j < np[a]; ++j) sacc += w * __ldg(x + par[a][j]);
-        xl[a] = sacc;
-    }
-    for (int a = 0; a < NC; ++a) {
-        float sacc = 0.0f;
-#pragma unroll
-        for (int b = 0; b < NC; ++b) sacc += (am * c_Mref[a * NC + b] + bk * c_Kref[a * NC + b]) * xl[b];
-        const float w = np[a] == 1 ? 1.0f : (np[a] == 2 ? 0.5f : 0.25f);
-        for (int j = 0; j < np[a]; ++j) atomicAdd(y + par[a][j], w * sacc);
-    }
-}
-
-// nodal psi''(phi~) with phi~ the mid-point average, and the lumped mass (FP32)
+// nodal psi''(phi~) with phi~ the mid-point average (FP32)
 template <class T>
 __global__ void ch_nodal_kernel(int64_t N, int NF, int fphi, const T* __restrict__ Uo, const T* __restrict__ Un,
-                                const double* __restrict__ nmass, float* __restrict__ psi2, float* __restrict__ ml) {
+                                float* __restrict__ psi2) {
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= N) return;
     const float ph = 0.5f * ((float)Uo[(size_t)n * NF + fphi] + (float)Un[(size_t)n * NF + fphi]);
     psi2[n] = 3.0f * ph * ph - 1.0f;
-    ml[n] = (float)nmass[n];
 }
 
-// rp = v_phi, rm = v_mu (strided FP64 input), a = rm / ml
-__global__ void ch_load_kernel(int64_t N, int NF, int fphi, const double* __restrict__ v, float* __restrict__ rp,
-                               float* __restrict__ rm, float* __restrict__ a, const float* __restrict__ ml) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    rp[n] = (float)v[(size_t)n * NF + fphi];
-    const float r = (float)v[(size_t)n * NF + fphi + 1];
-    rm[n] = r;
-    a[n] = r / ml[n];
+// What precond_setup found about its spectrum bounds: read with the next scalars the host waits for.
+chns_status pc_flags_fetch(Ctx& c) {
+    CHNS_CUDA(cudaMemcpyAsync(c.ws->hsc + MAXSC - 1, precond_flags(c.m), sizeof(unsigned int), cudaMemcpyDeviceToHost, c.s));
+    return CHNS_OK;
 }
-// t = rp + c * y
-__global__ void ch_axpy_kernel(int64_t N, const float* __restrict__ rp, const float* __restrict__ y, float c,
-                               float* __restrict__ t) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) t[n] = rp[n] + c * y[n];
+chns_status pc_flags_check(const Ctx& c) {
+    unsigned int f = 0;
+    std::memcpy(&f, c.ws->hsc + MAXSC - 1, sizeof(f));
+    if (f & 1u) { chns_set_error("pressure Schur spectrum bound is not finite"); return CHNS_ENAN; }
+    if (f & 2u) { chns_set_error("Cahn-Hilliard block spectrum bound is not finite"); return CHNS_ENAN; }
+    return CHNS_OK;
 }
-// z_phi = x, z_mu = psi2 x + Cn^2 (K x) / ml - 2 rm / ml
-template <class TO>
-__global__ void ch_store_kernel(int64_t N, int NF, int fphi, const float* __restrict__ x, const float* __restrict__ kx,
-                                const float* __restrict__ rm, const float* __restrict__ psi2,
-                                const float* __restrict__ ml, float cn2, TO* __restrict__ z) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    const float xv = x[n], il = 1.0f / ml[n];
-    z[(size_t)n * NF + fphi] = (TO)xv;
-    z[(size_t)n * NF + fphi + 1] = (TO)(psi2[n] * xv + cn2 * kx[n] * il - 2.0f * rm[n] * il);
-}
-
-__global__ void recip_kernel(float* __restrict__ d, int64_t n) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) d[i] = d[i] > 0.0f ? 1.0f / d[i] : 0.0f;
-}
-
-// r = v_p (strided input), x = 0, d = dinv r / theta, y = 0 (the first matvec's output)
-template <class TI>
-__global__ void cheb_init_kernel(int64_t N, int NF, int f, const TI* __restrict__ v, const float* __restrict__ dinv,
-                                 float* __restrict__ r, float* __restrict__ x, float* __restrict__ d, float* __restrict__ y,
-                                 float inv_theta) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    const float rv = (float)v[(size_t)n * NF + f];
-    r[n] = rv;
-    x[n] = 0.0f;
-    y[n] = 0.0f;
-    d[n] = inv_theta * dinv[n] * rv;
-}
-
-// x += d; r -= y; d = c1 d + c2 dinv r; y = 0 (ready for the next accumulating matvec)
-__global__ void cheb_step_kernel(int64_t N, const float* __restrict__ dinv, float* __restrict__ r, float* __restrict__ x,
-                                 float* __restrict__ d, float* __restrict__ y, float c1, float c2) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    x[n] += d[n];
-    const float rn = r[n] - y[n];
-    y[n] = 0.0f;
-    r[n] = rn;
-    d[n] = c1 * d[n] + c2 * dinv[n] * rn;
-}
-
-template <class TO>
-__global__ void cheb_final_kernel(int64_t N, int NF, int f, const float* __restrict__ x, const float* __restrict__ d,
-                                  TO* __restrict__ z) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) z[(size_t)n * NF + f] = (TO)(x[n] + d[n]);
-}
-
-
-// ---------------- geometric multigrid for the pressure Schur Laplacian ----------------
-// coarse element coefficients: the volume-weighted mean of the fine elements they hold
-__global__ void mg_restrict_ce_kernel(int64_t Ef, int D, const int32_t* __restrict__ fmap,
-                                      const int8_t* __restrict__ lev_f, const int8_t* __restrict__ lev_c,
-                                      const float* __restrict__ ce_f, float* __restrict__ ce_c) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= Ef) return;
-    const int c = fmap[e];
-    atomicAdd(ce_c + c, ldexpf(ce_f[e], -D * ((int)lev_f[e] - (int)lev_c[c])));
-}
-__global__ void mg_copy_kernel(int64_t N, const float* __restrict__ a, float* __restrict__ b) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) b[n] = a[n];
-}
-template <class TI>
-__global__ void mg_load_kernel(int64_t N, int NF, int f, const TI* __restrict__ v, float* __restrict__ b) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) b[n] = (float)v[(size_t)n * NF + f];
-}
-template <class TO>
-__global__ void mg_store_kernel(int64_t N, int NF, int f, const float* __restrict__ x, TO* __restrict__ z) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) z[(size_t)n * NF + f] = (TO)x[n];
-}
-// out += x + d (a Chebyshev correction added to an existing iterate)
-__global__ void cheb_final_add_kernel(int64_t N, const float* __restrict__ x, const float* __restrict__ d,
-                                      float* __restrict__ out) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) out[n] += x[n] + d[n];
-}
-
-// Chebyshev coefficients of the three-term recurrence on [alpha, beta] (degree deg)
-void cheb_coeffs(double alpha, double beta, int deg, std::vector<float>& c1, std::vector<float>& c2, float& inv_theta) {
-    const double theta = 0.5 * (beta + alpha), delta = 0.5 * (beta - alpha), sigma = theta / delta;
-    c1.assign(std::max(deg, 1), 0.0f);
-    c2.assign(std::max(deg, 1), 0.0f);
-    double rho = 1.0 / sigma;
-    for (int k = 0; k + 1 < deg; ++k) {
-        const double rn = 1.0 / (2.0 * sigma - rho);
-        c1[k] = (float)(rn * rho);
-        c2[k] = (float)(2.0 * rn / delta);
-        rho = rn;
-    }
-    inv_theta = (float)(1.0 / theta);
-}
-
-// One V-cycle for K x = b on level l (x overwritten), queued on stream st; returns the
-// number of kernels queued.  Each level: Chebyshev pre-smoothing from x = 0, residual,
-// restriction P^T, the coarser cycle, prolongation P added to x, residual, Chebyshev
-// post-smoothing added to x; the coarsest level is one long Chebyshev sweep.
-int mg_vcycle(MGHier* mg, int l, const float* ce0, cudaStream_t st) {
-    MGLevel& L = mg->lv[(size_t)l];
-    const float* ce = l == 0 ? ce0 : L.ce;
-    const int D = L.dm.dim;
-    const int gN = (int)((L.N + 255) / 256), gE = (int)((L.E + 255) / 256);
-    int nk = 0;
-    auto matvec = [&](const float* x, float* y, float sgn) {
-        if (D == 2) schur_matvec_kernel<2><<<gE, 256, 0, st>>>(L.dm, ce, x, y, sgn);
-        else schur_matvec_kernel<3><<<gE, 256, 0, st>>>(L.dm, ce, x, y, sgn);
-        ++nk;
-    };
-    auto cheb = [&](const float* in, float* out, bool add) {
-        cheb_init_kernel<float><<<gN, 256, 0, st>>>(L.N, 1, 0, in, L.dinv, L.cr, L.cx, L.cd, L.cy, L.inv_theta);
-        ++nk;
-        for (int k = 0; k + 1 < L.deg; ++k) {
-            matvec(L.cd, L.cy, 1.0f);
-            cheb_step_kernel<<<gN, 256, 0, st>>>(L.N, L.dinv, L.cr, L.cx, L.cd, L.cy, L.c1[(size_t)k], L.c2[(size_t)k]);
-            ++nk;
-        }
-        if (add) cheb_final_add_kernel<<<gN, 256, 0, st>>>(L.N, L.cx, L.cd, out);
-        else cheb_final_kernel<float><<<gN, 256, 0, st>>>(L.N, 1, 0, L.cx, L.cd, out);
-        ++nk;
-    };
-    if (l + 1 == (int)mg->lv.size()) {
-        cheb(L.b, L.x, false);
-        return nk;
-    }
-    MGLevel& C = mg->lv[(size_t)l + 1];
-    cheb(L.b, L.x, false);
-    mg_copy_kernel<<<gN, 256, 0, st>>>(L.N, L.b, L.t);
-    ++nk;
-    matvec(L.x, L.t, -1.0f);
-    transfer_apply_f32(C.P, true, false, L.t, C.b, st);
-    ++nk;
-    nk += mg_vcycle(mg, l + 1, ce0, st);
-    transfer_apply_f32(C.P, false, true, C.x, L.x, st);
-    ++nk;
-    mg_copy_kernel<<<gN, 256, 0, st>>>(L.N, L.b, L.t);
-    ++nk;
-    matvec(L.x, L.t, -1.0f);
-    cheb(L.t, L.x, true);
-    return nk;
-}
-
-// Pressure Schur-complement preconditioner (pc_type >= 1), shared by the Newton step and
-// the adjoint solve: set-up after the block-Jacobi build has written the element
-// coefficients ws->ce, then applies z_p = (approximation of S^{-1}) v_p, either a
-// Jacobi-Chebyshev polynomial of degree `degree` or one multigrid V-cycle (use_mg).
-struct SchurPC {
-    chns_mesh* m;
-    SolverWS* ws;
-    cudaStream_t s;
-    int degree;
-    bool use_mg;
-    int D, NF, gE, gN1, g;
-    SchurPC(chns_mesh* mm, SolverWS* w, cudaStream_t st, int deg, bool mg)
-        : m(mm), ws(w), s(st), degree(deg), use_mg(mg), D(mm->dm.dim), NF(mm->dm.nf),
-          gE((int)((mm->dm.E + 255) / 256)), gN1((int)((mm->dm.N + 255) / 256)), g(grid_for(w->n)) {}
-    chns_status setup() { return use_mg ? mg_setup() : cheb_setup(); }
-    chns_status cheb_setup() {
-        if (ws->kref_dim != D) {
-            float K[64], Mr[64];
-            kref_host(D, K);
-            mref_host(D, Mr);
-            CHNS_CUDA(cudaMemcpyToSymbolAsync(c_Kref, K, sizeof(float) * (1 << D) * (1 << D), 0,
-                                              cudaMemcpyHostToDevice, s));
-            CHNS_CUDA(cudaMemcpyToSymbolAsync(c_Mref, Mr, sizeof(float) * (1 << D) * (1 << D), 0,
-                                              cudaMemcpyHostToDevice, s));
-            ws->kref_dim = D;
-        }
-        const int64_t N = m->dm.N;
-        CHNS_CUDA(cudaMemsetAsync(ws->kdinv, 0, N * sizeof(float), s));
-        CHNS_CUDA(cudaMemsetAsync(ws->kbnd, 0, N * sizeof(float), s));
-        CHNS_CUDA(cudaMemsetAsync(ws->kmax, 0, sizeof(unsigned int), s));
-        if (D == 2) { schur_diag_kernel<2><<<gE, 256, 0, s>>>(m->dm, ws->ce, ws->kdinv, ws->kbnd); chns_count_launches(1); }
-        else { schur_diag_kernel<3><<<gE, 256, 0, s>>>(m->dm, ws->ce, ws->kdinv, ws->kbnd); chns_count_launches(1); }
-        { recip_kernel<<<gN1, 256, 0, s>>>(ws->kdinv, N); chns_count_launches(1); }
-        // The Chebyshev interval must not cut the top of the spectrum of D^{-1} K, where
-        // the polynomial would amplify.  Gershgorin with the row-sum bounds gives it for
-        // any positive D: 2 on a uniform mesh (off-diagonal stiffness entries are <= 0),
-        // more where hanging constraints fold positive weights into a row.
-        { gershgorin_max_kernel<<<g, 256, 0, s>>>(ws->kbnd, ws->kdinv, N, ws->kmax); chns_count_launches(1); }
-        unsigned int kbits = 0;
-        CHNS_CUDA(cudaMemcpyAsync(&ws->hsc[0], ws->kmax, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
-        CHNS_CUDA(cudaStreamSynchronize(s));
-        std::memcpy(&kbits, &ws->hsc[0], sizeof(unsigned int));
-        float kb;
-        std::memcpy(&kb, &kbits, sizeof(float));
-        if (!(kb > 0.0f) || !std::isfinite(kb)) { chns_set_error("pressure Schur spectrum bound is not finite"); return CHNS_ENAN; }
-        const double beta = 1.01 * (double)kb;
-        const double nside = std::ldexp(1.0, m->max_level);
-        const double ratio = std::max(16.0, nside * nside / 8.0);
-        const double alpha = beta / ratio;
-        const double theta = 0.5 * (beta + alpha), delta = 0.5 * (beta - alpha), sigma = theta / delta;
-        const int deg = degree;
-        ws->cheb_c1.assign(deg, 0.0f);
-        ws->cheb_c2.assign(deg, 0.0f);
-        double rho = 1.0 / sigma;
-        for (int k = 0; k + 1 < deg; ++k) {
-            const double rn = 1.0 / (2.0 * sigma - rho);
-            ws->cheb_c1[k] = (float)(rn * rho);
-            ws->cheb_c2[k] = (float)(2.0 * rn / delta);
-            rho = rn;
-        }
-        ws->cheb_inv_theta = (float)(1.0 / theta);
-        ws->schur_gen++;   // captured applies hold the old coefficients
-        return CHNS_OK;
-    }
-    chns_status mg_setup() {
-        if (ws->kref_dim != D) {
-            float K[64], Mr[64];
-            kref_host(D, K);
-            mref_host(D, Mr);
-            CHNS_CUDA(cudaMemcpyToSymbolAsync(c_Kref, K, sizeof(float) * (1 << D) * (1 << D), 0,
-                                              cudaMemcpyHostToDevice, s));
-            CHNS_CUDA(cudaMemcpyToSymbolAsync(c_Mref, Mr, sizeof(float) * (1 << D) * (1 << D), 0,
-                                              cudaMemcpyHostToDevice, s));
-            ws->kref_dim = D;
-        }
-        chns_status sb = mg_hier_build(m);
-        if (sb != CHNS_OK) return sb;
-        MGHier* mg = m->mg;
-        const int nl = (int)mg->lv.size();
-        for (int l = 1; l < nl; ++l) {
-            MGLevel& C = mg->lv[(size_t)l];
-            MGLevel& F = mg->lv[(size_t)l - 1];
-            CHNS_CUDA(cudaMemsetAsync(C.ce, 0, C.E * sizeof(float), s));
-            { mg_restrict_ce_kernel<<<(int)((F.E + 255) / 256), 256, 0, s>>>(F.E, D, C.fmap, F.dm.level, C.dm.level, l == 1 ? ws->ce : F.ce, C.ce); chns_count_launches(1); }
-        }
-        CHNS_CUDA(cudaMemsetAsync(mg->kmax, 0, nl * sizeof(unsigned int), s));
-        for (int l = 0; l < nl; ++l) {
-            MGLevel& L = mg->lv[(size_t)l];
-            const float* cel = l == 0 ? ws->ce : L.ce;
-            const int gEl = (int)((L.E + 255) / 256), gNl = (int)((L.N + 255) / 256);
-            CHNS_CUDA(cudaMemsetAsync(L.dinv, 0, L.N * sizeof(float), s));
-            CHNS_CUDA(cudaMemsetAsync(L.bnd, 0, L.N * sizeof(float), s));
-            if (D == 2) { schur_diag_kernel<2><<<gEl, 256, 0, s>>>(L.dm, cel, L.dinv, L.bnd); chns_count_launches(1); }
-            else { schur_diag_kernel<3><<<gEl, 256, 0, s>>>(L.dm, cel, L.dinv, L.bnd); chns_count_launches(1); }
-            { recip_kernel<<<gNl, 256, 0, s>>>(L.dinv, L.N); chns_count_launches(1); }
-            { gershgorin_max_kernel<<<grid_for(L.N), 256, 0, s>>>(L.bnd, L.dinv, L.N, mg->kmax + l); chns_count_launches(1); }
-        }
-        CHNS_CUDA(cudaGetLastError());
-        CHNS_CUDA(cudaMemcpyAsync(ws->hsc, mg->kmax, nl * sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
-        CHNS_CUDA(cudaStreamSynchronize(s));
-        for (int l = 0; l < nl; ++l) {
-            MGLevel& L = mg->lv[(size_t)l];
-            unsigned int kbits = 0;
-            std::memcpy(&kbits, reinterpret_cast<const unsigned char*>(ws->hsc) + l * sizeof(unsigned int),
-                        sizeof(unsigned int));
-            float kb;
-            std::memcpy(&kb, &kbits, sizeof(float));
-            if (!(kb > 0.0f) || !std::isfinite(kb)) { chns_set_error("multigrid spectrum bound is not finite"); return CHNS_ENAN; }
-            const double beta = 1.01 * (double)kb;
-            if (l + 1 < nl) {
-                // smoother: damp the upper part of the spectrum of D^{-1} K
-                L.deg = degree;
-                cheb_coeffs(beta / 10.0, beta, L.deg, L.c1, L.c2, L.inv_theta);
-            } else {
-                // coarsest level: one long sweep over the whole spectrum
-                const double nside = std::ldexp(1.0, L.mesh ? L.mesh->max_level : m->max_level);
-                L.deg = 16;
-                cheb_coeffs(beta / std::max(16.0, nside * nside / 8.0), beta, L.deg, L.c1, L.c2, L.inv_theta);
-            }
-        }
-        ws->schur_gen++;   // captured applies hold the old coefficients
-        return CHNS_OK;
-    }
-    template <class TI, class TO>
-    chns_status apply(const TI* vin, TO* zout) {
-        const int64_t N = m->dm.N;
-        // the apply is a sequence of short launches: replayed from a CUDA graph
-        auto enqueue = [&](cudaStream_t st) -> int {
-            if (use_mg) {
-                MGHier* mg = m->mg;
-                mg_load_kernel<TI><<<gN1, 256, 0, st>>>(N, NF, D, vin, mg->lv[0].b);
-                const int nv = mg_vcycle(mg, 0, ws->ce, st);
-                mg_store_kernel<TO><<<gN1, 256, 0, st>>>(N, NF, D, mg->lv[0].x, zout);
-                return nv + 2;
-            }
-            cheb_init_kernel<TI><<<gN1, 256, 0, st>>>(N, NF, D, vin, ws->kdinv, ws->cr, ws->cx, ws->cd, ws->cy, ws->cheb_inv_theta);
-            for (int k = 0; k + 1 < degree; ++k) {
-                if (D == 2) schur_matvec_kernel<2><<<gE, 256, 0, st>>>(m->dm, ws->ce, ws->cd, ws->cy);
-                else schur_matvec_kernel<3><<<gE, 256, 0, st>>>(m->dm, ws->ce, ws->cd, ws->cy);
-                cheb_step_kernel<<<gN1, 256, 0, st>>>(N, ws->kdinv, ws->cr, ws->cx, ws->cd, ws->cy, ws->cheb_c1[k], ws->cheb_c2[k]);
-            }
-            cheb_final_kernel<TO><<<gN1, 256, 0, st>>>(N, NF, D, ws->cx, ws->cd, zout);
-            return 2 + 2 * (degree - 1);
-        };
-        if (!ws->no_graphs) {
-            SolverWS::SchurGraph* hit = nullptr;
-            for (auto& g : ws->sgraph)
-                if (g.exec && g.gen == ws->schur_gen && g.vin == (const void*)vin && g.zout == (void*)zout &&
-                    g.to == sizeof(TO))
-                    hit = &g;
-            if (!hit) {
-                SolverWS::SchurGraph* slot = &ws->sgraph[0];
-                for (auto& g : ws->sgraph)
-                    if (!g.exec || g.gen != ws->schur_gen) { slot = &g; break; }
-                cudaGraphExec_t ex = nullptr;
-                cudaGraph_t gr = nullptr;
-                bool ok = ws->cap || cudaStreamCreateWithFlags(&ws->cap, cudaStreamNonBlocking) == cudaSuccess;
-                if (ok) ok = cudaStreamBeginCapture(ws->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-                int nk_cap = 0;
-                if (ok) {
-                    nk_cap = enqueue(ws->cap);
-                    ok = cudaStreamEndCapture(ws->cap, &gr) == cudaSuccess && gr != nullptr;
-                    if (ok) ok = cudaGraphInstantiate(&ex, gr, 0) == cudaSuccess;
-                    if (gr) cudaGraphDestroy(gr);
-                }
-                if (!ok) {
-                    (void)cudaGetLastError();   // capture unavailable: launch directly from now on
-                    ws->no_graphs = true;
-                } else {
-                    if (slot->exec) cudaGraphExecDestroy(slot->exec);
-                    slot->exec = ex;
-                    slot->vin = (const void*)vin;
-                    slot->zout = (void*)zout;
-                    slot->to = sizeof(TO);
-                    slot->gen = ws->schur_gen;
-                    slot->nk = nk_cap;
-                    hit = slot;
-                }
-            }
-            if (hit) {
-                CHNS_CUDA(cudaGraphLaunch(hit->exec, s));
-                chns_count_launches(hit->nk);
-                return CHNS_OK;
-            }
-        }
-        chns_count_launches(enqueue(s));
-        CHNS_CUDA(cudaGetLastError());
-        return CHNS_OK;
-    }
-};
 
 }  // namespace
 
@@ -1387,10 +818,20 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
     const int chblk = (o->pc_type == 2 || o->pc_type == 4) ? 1 : 0;
     const bool use_mg = o->pc_type >= 3;   // pressure Schur by a multigrid V-cycle
     const int pcmask = schur | (chblk << 1);
-    const int gE = (int)((m->dm.E + 255) / 256);
     const int gN1 = (int)((m->dm.N + 255) / 256);
-    SchurPC spc(m, ws, c.s, o->pc_degree, use_mg);
-    auto schur_apply_any = [&](auto vin, auto zout) -> chns_status { return spc.apply(vin, zout); };
+    PrecondSpec spec;
+    spec.schur = schur;
+    spec.mg = use_mg;
+    spec.ch = chblk;
+    spec.degree = o->pc_degree;
+    if (chblk) {
+        // Cahn-Hilliard block: S_phi ~ (1/dt)(M + eps K) M^{-1} (M + eps K), eps^2 = dt Cn/(2 Pe)
+        spec.dt = (float)p->dt;
+        spec.inv_pecn = (float)(1.0 / (p->Pe * p->Cn));
+        spec.cn2 = (float)(p->Cn * p->Cn);
+        spec.eps = (float)std::sqrt(p->dt * p->Cn / (2.0 * p->Pe));
+    }
+    if (schur && (st = precond_prepare(m, spec, c.s)) != CHNS_OK) return st;
     const int pin = p->pin_pressure;
     const int gN = (int)((m->dm.N + 127) / 128);
     chns_stats S;
@@ -1405,80 +846,6 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
     std::vector<double> H((size_t)(mres + 1) * mres), cs(mres), sn(mres), gv(mres + 1), y(mres);
     double r0 = 0.0, rn = 0.0;
     chns_status result = CHNS_OK;
-    // Cahn-Hilliard block: S_phi ~ (1/dt)(M + eps K) M^{-1} (M + eps K), eps^2 = dt Cn/(2 Pe)
-    const float span = (float)(m->dm.hi - m->dm.lo);
-    const int CH_DEG = 8;
-    auto mk = [&](float alpha, float beta, const float* x, float* y) -> chns_status {
-        CHNS_CUDA(cudaMemsetAsync(y, 0, m->dm.N * sizeof(float), c.s));
-        if (D == 2) { mk_kernel<2, false><<<gE, 256, 0, c.s>>>(m->dm, span, alpha, beta, x, y); chns_count_launches(1); }
-        else { mk_kernel<3, false><<<gE, 256, 0, c.s>>>(m->dm, span, alpha, beta, x, y); chns_count_launches(1); }
-        return CHNS_OK;
-    };
-    auto ch_setup = [&](const void* Uo_any, const void* Un_any) -> chns_status {
-        const int64_t N = m->dm.N;
-        if (mixed) { ch_nodal_kernel<float><<<gN1, 256, 0, c.s>>>(N, NF, D + 1, (const float*)Uo_any, (const float*)Un_any, m->d_nmass, ws->ch_psi2, ws->ch_ml); chns_count_launches(1); }
-        else { ch_nodal_kernel<double><<<gN1, 256, 0, c.s>>>(N, NF, D + 1, (const double*)Uo_any, (const double*)Un_any, m->d_nmass, ws->ch_psi2, ws->ch_ml); chns_count_launches(1); }
-        ws->ch_eps = (float)std::sqrt(p->dt * p->Cn / (2.0 * p->Pe));
-        CHNS_CUDA(cudaMemsetAsync(ws->ch_dinv, 0, N * sizeof(float), c.s));
-        CHNS_CUDA(cudaMemsetAsync(ws->kbnd, 0, N * sizeof(float), c.s));
-        CHNS_CUDA(cudaMemsetAsync(ws->kmax, 0, sizeof(unsigned int), c.s));
-        if (D == 2) { mk_kernel<2, true><<<gE, 256, 0, c.s>>>(m->dm, span, 1.0f, ws->ch_eps, nullptr, ws->ch_dinv, ws->kbnd); chns_count_launches(1); }
-        else { mk_kernel<3, true><<<gE, 256, 0, c.s>>>(m->dm, span, 1.0f, ws->ch_eps, nullptr, ws->ch_dinv, ws->kbnd); chns_count_launches(1); }
-        { recip_kernel<<<gN1, 256, 0, c.s>>>(ws->ch_dinv, N); chns_count_launches(1); }
-        // top of the spectrum of D^{-1}(M + eps K): Gershgorin with the row-sum bounds
-        // (3.375 for the Q1 mass on a uniform 3D mesh, 2 for the stiffness)
-        { gershgorin_max_kernel<<<c.g, 256, 0, c.s>>>(ws->kbnd, ws->ch_dinv, N, ws->kmax); chns_count_launches(1); }
-        CHNS_CUDA(cudaGetLastError());
-        unsigned int kbits = 0;
-        CHNS_CUDA(cudaMemcpyAsync(&ws->hsc[0], ws->kmax, sizeof(unsigned int), cudaMemcpyDeviceToHost, c.s));
-        CHNS_CUDA(cudaStreamSynchronize(c.s));
-        std::memcpy(&kbits, &ws->hsc[0], sizeof(unsigned int));
-        float kb;
-        std::memcpy(&kb, &kbits, sizeof(float));
-        if (!(kb > 0.0f) || !std::isfinite(kb)) { chns_set_error("Cahn-Hilliard block spectrum bound is not finite"); return CHNS_ENAN; }
-        const double beta = 1.01 * (double)kb, alpha = 0.05;
-        const double theta = 0.5 * (beta + alpha), delta = 0.5 * (beta - alpha), sigma = theta / delta;
-        ws->ch_c1.assign(CH_DEG, 0.0f);
-        ws->ch_c2.assign(CH_DEG, 0.0f);
-        double rho = 1.0 / sigma;
-        for (int k = 0; k + 1 < CH_DEG; ++k) {
-            const double rn = 1.0 / (2.0 * sigma - rho);
-            ws->ch_c1[k] = (float)(rn * rho);
-            ws->ch_c2[k] = (float)(2.0 * rn / delta);
-            rho = rn;
-        }
-        ws->ch_inv_theta = (float)(1.0 / theta);
-        return CHNS_OK;
-    };
-    // out = Chebyshev approximation of (M + eps K)^{-1} in (contiguous FP32)
-    auto ch_cheb = [&](const float* in, float* out) -> chns_status {
-        const int64_t N = m->dm.N;
-        { cheb_init_kernel<float><<<gN1, 256, 0, c.s>>>(N, 1, 0, in, ws->ch_dinv, ws->cr, ws->cx, ws->cd, ws->cy, ws->ch_inv_theta); chns_count_launches(1); }
-        for (int k = 0; k + 1 < CH_DEG; ++k) {
-            chns_status s2 = mk(1.0f, ws->ch_eps, ws->cd, ws->cy);
-            if (s2 != CHNS_OK) return s2;
-            { cheb_step_kernel<<<gN1, 256, 0, c.s>>>(N, ws->ch_dinv, ws->cr, ws->cx, ws->cd, ws->cy, ws->ch_c1[k], ws->ch_c2[k]); chns_count_launches(1); }
-        }
-        { cheb_final_kernel<float><<<gN1, 256, 0, c.s>>>(N, 1, 0, ws->cx, ws->cd, out); chns_count_launches(1); }
-        CHNS_CUDA(cudaGetLastError());
-        return CHNS_OK;
-    };
-    auto ch_apply_any = [&](const double* v, auto zout) -> chns_status {
-        using TO = std::remove_pointer_t<decltype(zout)>;
-        const int64_t N = m->dm.N;
-        chns_status s2;
-        { ch_load_kernel<<<gN1, 256, 0, c.s>>>(N, NF, D + 1, v, ws->ch_b, ws->ch_rm, ws->ch_a, ws->ch_ml); chns_count_launches(1); }
-        if ((s2 = mk(0.0f, 1.0f, ws->ch_a, ws->ch_c)) != CHNS_OK) return s2;                 // K M_L^{-1} r_mu
-        { ch_axpy_kernel<<<gN1, 256, 0, c.s>>>(N, ws->ch_b, ws->ch_c, (float)(1.0 / (p->Pe * p->Cn)), ws->ch_b); chns_count_launches(1); }
-        if ((s2 = ch_cheb(ws->ch_b, ws->ch_a)) != CHNS_OK) return s2;                      // (M + eps K)^{-1} t
-        if ((s2 = mk(1.0f, 0.0f, ws->ch_a, ws->ch_c)) != CHNS_OK) return s2;                // M s
-        { axpbyf_kernel<<<gN1, 256, 0, c.s>>>((float)p->dt, ws->ch_c, N); chns_count_launches(1); }
-        if ((s2 = ch_cheb(ws->ch_c, ws->ch_a)) != CHNS_OK) return s2;                      // dphi
-        if ((s2 = mk(0.0f, 1.0f, ws->ch_a, ws->ch_c)) != CHNS_OK) return s2;                // K dphi
-        { ch_store_kernel<TO><<<gN1, 256, 0, c.s>>>(N, NF, D + 1, ws->ch_a, ws->ch_c, ws->ch_rm, ws->ch_psi2, ws->ch_ml, (float)(p->Cn * p->Cn), zout); chns_count_launches(1); }
-        CHNS_CUDA(cudaGetLastError());
-        return CHNS_OK;
-    };
     // one classical Gram-Schmidt pass against V_0..V_{k-1}: h -> hdev[0..k), |w|^2 before
     // -> nrm_before, |w|^2 after -> nrm_after (all device scalars); with pred, every kernel
     // of the pass returns at once when pred[0] == 0
@@ -1515,12 +882,14 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
             { pc_invert_kernel<double, double><<<gN, 128, 0, c.s>>>(m->dm, ws->Pblk64, ws->Pinv64, pin, ws->S, ws->Sd, pcmask); chns_count_launches(1); }
         }
         CHNS_CUDA(cudaGetLastError());
-        if (schur) {
-            chns_status st3 = spc.setup();
-            if (st3 != CHNS_OK) return st3;
-        }
         if (chblk) {
-            chns_status st3 = mixed ? ch_setup(ws->Uo32, ws->Us32) : ch_setup(U_old, U);
+            if (mixed) ch_nodal_kernel<float><<<gN1, 256, 0, c.s>>>(m->dm.N, NF, D + 1, ws->Uo32, ws->Us32, ws->ch_psi2);
+            else ch_nodal_kernel<double><<<gN1, 256, 0, c.s>>>(m->dm.N, NF, D + 1, U_old, U, ws->ch_psi2);
+            chns_count_launches(1);
+        }
+        if (schur) {
+            chns_status st3 = precond_setup(m, spec, ws->ce, ws->ch_psi2, c.s);
+            if (st3 == CHNS_OK) st3 = pc_flags_fetch(c);
             if (st3 != CHNS_OK) return st3;
         }
         CHNS_CUDA(cudaEventRecord(ws->ev[3], c.s));
@@ -1547,6 +916,7 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
         }
         { scale_vec_kernel<double><<<c.g, 256, 0, c.s>>>(ws->R, ws->S0, ws->SR, c.n); chns_count_launches(1); }
         if ((st = dot_host(c, ws->SR, ws->SR, &rn)) != CHNS_OK) return st;
+        if (schur && (st = pc_flags_check(c)) != CHNS_OK) return st;
         unsigned int flag = 0;
         CHNS_CUDA(cudaMemcpy(&flag, m->d_flags, sizeof(unsigned int), cudaMemcpyDeviceToHost));
         rn = std::sqrt(rn);
@@ -1576,6 +946,7 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
         {
             double bb;
             if ((st = dot_host(c, ws->w, ws->w, &bb)) != CHNS_OK) return st;
+            if (schur && (st = pc_flags_check(c)) != CHNS_OK) return st;
             rnorm = std::sqrt(bb);
         }
         const double bnorm_s = rnorm;
@@ -1609,8 +980,7 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
             { unscale_kernel<<<c.g, 256, 0, c.s>>>(Vj, ws->Sd, ws->SR, c.n); chns_count_launches(1); }
             if (mixed) {
                 { pc_apply_kernel<float, float><<<gN, 128, 0, c.s>>>(m->dm.N, NF, ws->Pinv32, ws->SR, ws->z32); chns_count_launches(1); }
-                if (schur && (st = schur_apply_any((const double*)ws->SR, ws->z32)) != CHNS_OK) return st;
-                if (chblk && (st = ch_apply_any((const double*)ws->SR, ws->z32)) != CHNS_OK) return st;
+                if (schur && (st = precond_apply(m, spec, ws->SR, ws->z32, c.s)) != CHNS_OK) return st;
                 if (pin == 2) pmean(ws->z32);
                 CHNS_CUDA(cudaEventRecord(E[5], c.s));
                 CHNS_CUDA(cudaEventRecord(E[0], c.s));
@@ -1622,8 +992,7 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
                     { scale_vec_kernel<float><<<c.g, 256, 0, c.s>>>(ws->y32, ws->S, ws->w, c.n); chns_count_launches(1); }
             } else {
                 { pc_apply_kernel<double, double><<<gN, 128, 0, c.s>>>(m->dm.N, NF, ws->Pinv64, ws->SR, ws->z64); chns_count_launches(1); }
-                if (schur && (st = schur_apply_any((const double*)ws->SR, ws->z64)) != CHNS_OK) return st;
-                if (chblk && (st = ch_apply_any((const double*)ws->SR, ws->z64)) != CHNS_OK) return st;
+                if (schur && (st = precond_apply(m, spec, ws->SR, ws->z64, c.s)) != CHNS_OK) return st;
                 if (pin == 2) pmean(ws->z64);
                 CHNS_CUDA(cudaEventRecord(E[5], c.s));
                 CHNS_CUDA(cudaEventRecord(E[0], c.s));
@@ -1744,8 +1113,7 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
                 { pc_apply_kernel<float, double><<<gN, 128, 0, c.s>>>(m->dm.N, NF, ws->Pinv32, ws->SR, ws->z64); chns_count_launches(1); }
             else
                 { pc_apply_kernel<double, double><<<gN, 128, 0, c.s>>>(m->dm.N, NF, ws->Pinv64, ws->SR, ws->z64); chns_count_launches(1); }
-            if (schur && (st = schur_apply_any((const double*)ws->SR, ws->z64)) != CHNS_OK) return st;
-            if (chblk && (st = ch_apply_any((const double*)ws->SR, ws->z64)) != CHNS_OK) return st;
+            if (schur && (st = precond_apply(m, spec, ws->SR, ws->z64, c.s)) != CHNS_OK) return st;
             { axpy_kernel<<<c.g, 256, 0, c.s>>>(1.0, ws->z64, ws->dU, c.n); chns_count_launches(1); }
             CHNS_CUDA(cudaGetLastError());
             if (done || kry >= o->max_krylov) break;
@@ -1955,7 +1323,11 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
     // the pressure Schur approximation is symmetric, so J^T takes it as J does; the
     // Cahn-Hilliard block of pc_type 2 / 4 is not used here
     const bool schur = o->pc_type >= 1;
-    SchurPC spc(m, ws, c.s, o->pc_degree, o->pc_type >= 3);
+    PrecondSpec spec;
+    spec.schur = schur;
+    spec.mg = o->pc_type >= 3;
+    spec.degree = o->pc_degree;
+    if (schur && (st = precond_prepare(m, spec, c.s)) != CHNS_OK) return st;
     const int gN = (int)((m->dm.N + 127) / 128);
     const int nbk = c.g < 1024 ? c.g : 1024;
     chns_stats S;
@@ -1966,7 +1338,10 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
                               : pc_build_launch<3, double>(m, pc, U_old, U_new, ws->Pblk64, ws->ce, c.s);
     CHNS_CUDA(ce);
     { pc_invert_kernel<double, double><<<gN, 128, 0, c.s>>>(m->dm, ws->Pblk64, ws->Pinv64, pin, ws->S, ws->Sd, schur ? 1 : 0); chns_count_launches(1); }
-    if (schur && (st = spc.setup()) != CHNS_OK) return st;
+    if (schur) {
+        if ((st = precond_setup(m, spec, ws->ce, nullptr, c.s)) != CHNS_OK) return st;
+        if ((st = pc_flags_fetch(c)) != CHNS_OK) return st;
+    }
     // pin mode 2: J' = J + u m_p^T / |Omega| with u = |diag J| on the pressure rows is
     // nonsingular, and J'^T lambda = P^T g has the solution of J^T lambda = P^T g with
     // u^T lambda = 0 (GMRES on the singular J^T drifts along its null vector)
@@ -1987,6 +1362,7 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
     CHNS_CUDA(cudaGetLastError());
     double bb;
     if ((st = dot_host(c, b, b, &bb)) != CHNS_OK) return st;
+    if (schur && (st = pc_flags_check(c)) != CHNS_OK) return st;
     const double bnorm = std::sqrt(bb);
     CHNS_CUDA(cudaMemsetAsync(lambda, 0, c.n * sizeof(double), c.s));
     S.res0 = bnorm;
@@ -2007,7 +1383,11 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
             for (; j < mres && kry < o->max_krylov; ++j, ++kry) {
                 double* Vj = ws->V + (size_t)j * c.n;
                 { pc_apply_T_kernel<double><<<gN, 128, 0, c.s>>>(m->dm.N, NF, ws->Pinv64, Vj, ws->z64); chns_count_launches(1); }
-                if (schur && (st = spc.apply((const double*)Vj, ws->z64)) != CHNS_OK) return st;
+                if (schur) {
+                    // from a fixed vector, so that one captured graph serves every j
+                    { copy64_kernel<<<c.g, 256, 0, c.s>>>(Vj, ws->SR, c.n); chns_count_launches(1); }
+                    if ((st = precond_apply(m, spec, ws->SR, ws->z64, c.s)) != CHNS_OK) return st;
+                }
                 CHNS_CUDA(launch_vjp(m, pc, U_old, U_new, ws->z64, ws->w, nullptr, nullptr, pin, c.s));
                 if (pin == 2) add_pmean_T(ws->z64, ws->w);
                 S.jvp_calls++;
@@ -2058,7 +1438,7 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
             CHNS_CUDA(cudaMemcpyAsync(ws->sc, ws->hsc, k * sizeof(double), cudaMemcpyHostToDevice, c.s));
             { combine_kernel<<<c.g, 256, 0, c.s>>>(ws->V, c.n, k, ws->sc, ws->t64, c.n); chns_count_launches(1); }
             { pc_apply_T_kernel<double><<<gN, 128, 0, c.s>>>(m->dm.N, NF, ws->Pinv64, ws->t64, ws->z64); chns_count_launches(1); }
-            if (schur && (st = spc.apply((const double*)ws->t64, ws->z64)) != CHNS_OK) return st;
+            if (schur && (st = precond_apply(m, spec, ws->t64, ws->z64, c.s)) != CHNS_OK) return st;
             { axpy_kernel<<<c.g, 256, 0, c.s>>>(1.0, ws->z64, lambda, c.n); chns_count_launches(1); }
             CHNS_CUDA(cudaGetLastError());
             if (done || kry >= o->max_krylov) break;

@@ -1,0 +1,76 @@
+"""The assembled preconditioners of the Newton step over the forms that take different routes: a
+mesh whose whole polynomial or V-cycle runs in one block, mid-size levels with four lanes per row,
+hanging rows, smoother degrees 2 (one pass) and above, both precisions, 2D and 3D, and the
+Cahn-Hilliard block.  The preconditioner must not change the converged step (row-equilibrated
+residual <= 1e-11 of the first: 1e-9 in the state, as between the mixed and the FP64 step), and
+the pressure approximations must do their work: fewer GMRES iterations than plain block-Jacobi
+(the Cahn-Hilliard block does not claim that on meshes of this size); each spec again after another
+one (graphs and descriptions are rebuilt) takes the first one's iterations."""
+import os
+
+import numpy as np
+import pytest
+import torch
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def chns():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    import paper_2009_06628_gb300 as chns
+    if not os.path.exists(chns.LIB_PATH):
+        from paper_2009_06628_gb300 import build
+        build.build()
+    chns.load()
+    return chns
+
+
+def problem(chns, dim, leaves, level, cfg_name, **over):
+    cfg = synth.config_params(cfg_name)
+    cfg.update(over)
+    gm = chns.Mesh(dim, level, leaves)
+    x = gm.node_x()
+    U = np.zeros((gm.N, dim + 3))
+    U[:, dim + 1] = synth.drop_phi(x, [[0.5] * dim], [0.25], cfg["Cn"], noise=1e-3, seed=3)
+    U[:, :dim] = synth.fourier_velocity(x, 6, 4, 0.1)
+    U[np.any((x <= 0.0) | (x >= 1.0), axis=1), :dim] = 0.0
+    U = torch.tensor(U, device="cuda")
+    prm = chns.Params.make(**cfg)
+    chns.initial_mu(gm, prm, U)
+    return gm, prm, U
+
+
+@pytest.mark.parametrize("dim,kind,level", [(2, "uniform", 3), (2, "band", 6), (3, "uniform", 2), (3, "band", 4),
+                                            (3, "band", 5)])
+def test_preconditioners_keep_the_step(chns, dim, kind, level):
+    leaves = synth.uniform_leaves(dim, level) if kind == "uniform" else \
+        synth.sphere_band_leaves(dim, 2, level, [[0.5] * dim], [0.25], 0.04)
+    gm, prm, U0 = problem(chns, dim, leaves, level, "drop3d" if dim == 3 else "drop2d", Cn=0.05, rho_ratio=5.0,
+                          eta_ratio=3.0, Fr=1.0)
+    assert kind == "uniform" or gm.H > 0
+    kw = dict(rtol=1e-11, atol=1e-16, restart=60, max_krylov=6000, max_newton=20)
+    ref, s0 = chns.newton_step(gm, prm, chns.SolverOpts.make(precision=0, pc_type=0, krylov_rtol=1e-6, **kw), U0)
+    rel = lambda a: float((a - ref).norm() / ref.norm())
+    first = {}
+    for pc, deg in ((1, 2), (1, 16), (2, 8), (3, 2), (3, 3), (4, 2), (4, 5), (1, 16), (4, 2)):
+        for prec in (1, 0):
+            o = chns.SolverOpts.make(precision=prec, pc_type=pc, pc_degree=deg, krylov_rtol=1e-4, **kw)
+            U1, st = chns.newton_step(gm, prm, o, U0)
+            assert st.reason == 0 and rel(U1) <= 1e-9, (pc, deg, prec, rel(U1))
+            if pc in (1, 3) and gm.N > 100:
+                assert st.krylov_its < s0.krylov_its, (pc, deg, prec, st.krylov_its, s0.krylov_its)
+            key = (pc, deg, prec)
+            assert abs(first.setdefault(key, st.krylov_its) - st.krylov_its) <= 2, key
+
+
+def test_not_finite_coefficients_are_reported(chns):
+    gm, prm, U0 = problem(chns, 2, synth.uniform_leaves(2, 3), 3, "drop2d")
+    U0[5, 3] = float("nan")
+    for pc in (1, 3):
+        with pytest.raises(chns.ChnsError) as e:
+            chns.newton_step(gm, prm, chns.SolverOpts.make(precision=1, pc_type=pc, pc_degree=4), U0)
+        assert e.value.name == "CHNS_ENAN" and "bound" in str(e.value)
