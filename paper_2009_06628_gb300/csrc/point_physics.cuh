@@ -308,6 +308,90 @@ __device__ __forceinline__ void pw_tangent(const PwState<D, S>& P, const PwIn<D,
     F0[D + 2] = fma3(fma3(mul2(splat<S>(3.0), P.phi), P.phi, splat<S>(-1.0)), X.phi, neg1(dmu));
 }
 
+// Tangent for a basis function of one field alone (field F: v_F, p = D, mu = D + 2; for phi use
+// pw_tangent): n its averaged value, g[k] its D_k derivatives.  The terms that such a tangent
+// does not move are left out, which is more than half of them.
+template <int D, class S, int F>
+__device__ __forceinline__ void pw_unit(const PwState<D, S>& P, S n, const S g[D], const PwConst<S>& c,
+                                        const PwLevel<S>& L, const S sg[D], S F0[D + 3], S F1[D + 3][D]) {
+    const S z0 = splat<S>(0.0);
+    const S w = mul2(L.ct, P.tm), tm2 = mul2(P.tm, P.tm);
+    S dRm[D], dkh[D], dS[D], dSh[D], dbh[D], ddiag = z0, dtmr = z0, dcc = z0, dvh = z0;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        F0[i] = z0;
+        dkh[i] = z0;
+        F1[D + 2][i] = z0;
+    }
+    F0[D] = F0[D + 1] = F0[D + 2] = z0;
+    if constexpr (F < D) {
+        dvh = mul2(sg[F], n);
+        dkh[F] = mul2(P.rho, dvh);
+        const S dbase = mul2(mul2(P.rho, c.td), n);
+        const S dRc = mul2(sg[F], g[F]);
+        const S drad = mul2(mul2(c.gk, P.irho), fma3(dvh, P.kh[F], mul2(P.vh[F], dkh[F])));
+        const S dtp = neg1(mul2(mul2(c.gk, mul2(mul2(P.tp, P.tp), P.tp)), mul2(P.vh[F], dvh)));
+        dtmr = mul2(mul2(mul2(splat<S>(-0.5), mul2(tm2, P.tm)), drad), P.irho);
+        dcc = fma3(dtp, P.Rphi, mul2(P.tp, fma3(P.phi, dRc, mul2(dvh, P.gq[F]))));
+        ddiag = fma3(mul2(w, P.rad), mul2(P.rho, dRc), mul2(mul2(mul2(splat<S>(0.5), w), mul2(P.rho, P.Rc)), drad));
+        S r = dbase, f = dbase;
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            r = fma3(P.keh[j], g[j], r);
+            f = fma3(P.bh[j], g[j], f);
+        }
+#pragma unroll
+        for (int i = 0; i < D; ++i) dRm[i] = i == F ? fma3(dkh[F], P.gv[i][F], r) : mul2(dkh[F], P.gv[i][F]);
+        F0[F] = f;
+        F0[D] = add2(dRc, dRc);
+    } else if constexpr (F == D) {
+#pragma unroll
+        for (int i = 0; i < D; ++i) dRm[i] = mul2(mul2(sg[i], c.inv_We), g[i]);
+        ddiag = neg1(mul2(c.inv_We, n));
+    } else {
+        S dvk = z0;
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            dkh[j] = mul2(L.nak, g[j]);
+            dvk = fma3(P.vh[j], dkh[j], dvk);
+        }
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            S r = z0;
+#pragma unroll
+            for (int j = 0; j < D; ++j) r = fma3(dkh[j], P.gv[i][j], r);
+            dRm[i] = r;
+        }
+        const S drad = mul2(mul2(c.gk, P.irho), dvk);
+        dtmr = mul2(mul2(mul2(splat<S>(-0.5), mul2(tm2, P.tm)), drad), P.irho);
+        ddiag = mul2(mul2(mul2(splat<S>(0.5), w), mul2(P.rho, P.Rc)), drad);
+        F0[D + 2] = neg1(n);
+    }
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+        dS[j] = F == D ? mul2(P.tmr, dRm[j]) : fma3(P.tmr, dRm[j], mul2(dtmr, P.Rm[j]));
+        dSh[j] = mul2(sg[j], dS[j]);
+        dbh[j] = nfma3(P.rho, dSh[j], dkh[j]);
+    }
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            F0[i] = fma3(dbh[j], P.gv[i][j], F0[i]);
+            S t = fma3(P.Sv[i], dbh[j], mul2(dS[i], P.bh[j]));
+            if (F < D && i == F) t = fma3(P.EK, g[j], t);
+            if (i == j) t = fma3(sg[i], ddiag, t);
+            F1[i][j] = t;
+        }
+        F1[D][i] = dSh[i];
+        S t = mul2(dSh[i], P.phi);
+        if (F < D) t = fma3(P.vh[i], dcc, t);
+        if (F < D && i == F) t = fma3(dvh, P.cc, t);
+        if (F == D + 2) t = fma3(L.km, g[i], t);
+        F1[D + 1][i] = t;
+    }
+}
+
 // Adjoint: F0, F1 hold the cotangents of the fluxes (value and D_k gradient of the test field);
 // returns the cotangents of the inputs in Xb (Xb.a, Xb.pdt those of the time differences), of
 // p/We, mu and div v^{k+1}, and of Cn.  iCn = 1/Cn.

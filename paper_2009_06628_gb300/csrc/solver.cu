@@ -20,8 +20,8 @@
 #include <utility>
 #include <vector>
 
+#include "block_jacobi.h"
 #include "chns_internal.h"
-#include "pointwise.cuh"
 #include "precond.h"
 #include "reduce.cuh"
 
@@ -355,14 +355,6 @@ int grid_for(int64_t n) {
 }
 
 // ---------------- block-Jacobi preconditioner ----------------
-// Diagonal n_f x n_f block of every independent node, from the element-corner self
-// blocks d r_e[a] / d u_e[a] (forward mode with unit tangents).  Hanging corners are
-// skipped: the preconditioner is approximate there (it only affects convergence).
-template <int D, class T>
-__global__ void __launch_bounds__(128) pc_build_kernel(DevMesh m, PCst<T> c, T inv_dt, const T* __restrict__ Uo,
-                                                       const T* __restrict__ Un, T* __restrict__ blk,
-                                                       float* __restrict__ ce, double ce_scale);
-
 constexpr double GPc = 0.78867513459481288225, GMc = 0.21132486540518711775;
 
 template <int D, class T>
@@ -392,142 +384,6 @@ __device__ __forceinline__ PB<D, T> pbasis(int a, int q, T inv_h) {
         b.d2N[2] = f[0] * s[1] * s[2];
     }
     return b;
-}
-
-template <int D, class T>
-__global__ void __launch_bounds__(128) pc_build_kernel(DevMesh m, PCst<T> c, T inv_dt, const T* __restrict__ Uo,
-                                                       const T* __restrict__ Un, T* __restrict__ blk,
-                                                       float* __restrict__ ce, double ce_scale) {
-    constexpr int NC = 1 << D, NF = D + 3, NH = (D == 2) ? 1 : 3, EPB = 128 / NC;
-    __shared__ T s_ut[EPB][NC][NF], s_dd[EPB][NC][D + 1], s_ps[EPB][NC];
-    __shared__ int s_node[EPB][NC];
-    __shared__ unsigned char s_mask[EPB][NC];
-    const int le = threadIdx.x / NC, t = threadIdx.x % NC;
-    const int64_t e = (int64_t)blockIdx.x * EPB + le;
-    const bool valid = e < m.E;
-    T inv_h = T(1), detJ = T(0);
-    if (valid) {
-        const int ent = m.e2n[e * NC + t];
-        int p[4] = {0, 0, 0, 0}, np = 1;
-        if (ent >= 0) {
-            p[0] = ent;
-        } else {
-            const int4 hp = reinterpret_cast<const int4*>(m.hang)[-ent - 1];
-            p[0] = hp.x;
-            p[1] = hp.y;
-            p[2] = hp.z;
-            p[3] = hp.w;
-            np = hp.z < 0 ? 2 : 4;
-        }
-        const T wt = np == 1 ? T(1) : (np == 2 ? T(0.5) : T(0.25));
-        T so[NF], sn[NF], ps = T(0);
-        unsigned mask = 0;
-        for (int f = 0; f < NF; ++f) so[f] = sn[f] = T(0);
-        for (int j = 0; j < np; ++j) {
-            T o[NF], n[NF];
-            for (int f = 0; f < NF; ++f) {
-                o[f] = Uo[(size_t)p[j] * NF + f];
-                n[f] = Un[(size_t)p[j] * NF + f];
-                so[f] += wt * o[f];
-                sn[f] += wt * n[f];
-            }
-            const T avg = T(0.5) * (o[D + 1] + n[D + 1]);
-            if (avg <= T(1) && avg >= T(-1)) mask |= 1u << j;
-            ps += wt * (avg > T(1) ? T(1) : (avg < T(-1) ? T(-1) : avg));
-        }
-        for (int f = 0; f < NF; ++f) s_ut[le][t][f] = T(0.5) * (so[f] + sn[f]);
-        for (int i = 0; i < D; ++i) s_dd[le][t][i] = sn[i] - so[i];
-        s_dd[le][t][D] = sn[D + 1] - so[D + 1];
-        s_ps[le][t] = ps;
-        s_node[le][t] = ent;
-        s_mask[le][t] = (unsigned char)(mask & 1u);
-        const T h = T(ldexp(m.hi - m.lo, -(int)m.level[e]));
-        inv_h = T(1) / h;
-        detJ = (D == 2) ? T(0.25) * h * h : T(0.125) * h * h * h;
-    }
-    __syncwarp();
-    if (!valid) return;  // the remaining code uses only shuffles within the element's lanes
-    const int q = t;
-    const T g = T(4) * inv_h * inv_h;
-    // primal inputs at Gauss point q
-    QPIn<D, T> X;
-    {
-        X.p = X.phi = X.mu = X.phidt = X.divnew = X.ps = T(0);
-        for (int k = 0; k < D; ++k) {
-            X.v[k] = X.gp[k] = X.gphi[k] = X.gmu[k] = X.vdt[k] = X.gps[k] = T(0);
-            for (int j = 0; j < D; ++j) X.gv[k][j] = T(0);
-        }
-        for (int k = 0; k < NH; ++k) X.H[k] = T(0);
-        for (int a = 0; a < NC; ++a) {
-            const PB<D, T> b = pbasis<D, T>(a, q, inv_h);
-            const T* u = s_ut[le][a];
-            for (int i = 0; i < D; ++i) {
-                X.v[i] += b.N * u[i];
-                for (int k = 0; k < D; ++k) X.gv[i][k] += b.dN[k] * u[i];
-                X.vdt[i] += b.N * s_dd[le][a][i];
-                X.divnew += b.dN[i] * (u[i] + T(0.5) * s_dd[le][a][i]);
-            }
-            X.p += b.N * u[D];
-            X.phi += b.N * u[D + 1];
-            X.mu += b.N * u[D + 2];
-            for (int k = 0; k < D; ++k) {
-                X.gp[k] += b.dN[k] * u[D];
-                X.gphi[k] += b.dN[k] * u[D + 1];
-                X.gmu[k] += b.dN[k] * u[D + 2];
-                X.gps[k] += b.dN[k] * s_ps[le][a];
-            }
-            for (int k = 0; k < NH; ++k) X.H[k] += b.d2N[k] * u[D + 1];
-            X.phidt += b.N * s_dd[le][a][D];
-            X.ps += b.N * s_ps[le][a];
-        }
-        for (int i = 0; i < D; ++i) X.vdt[i] *= inv_dt;
-        X.phidt *= inv_dt;
-    }
-    const unsigned lanes = ((1u << NC) - 1u) << ((threadIdx.x & 31) & ~(NC - 1));
-    {
-        // coefficient of the pressure Schur-complement approximation on this element:
-        // dt/(2 We) times the mean of 1/rho(phi*) over the Gauss points
-        T ir = T(1) / (c.alpha * X.ps + c.beta);
-        for (int off = NC / 2; off > 0; off >>= 1) ir += __shfl_xor_sync(lanes, ir, off);
-        if (q == 0) ce[e] = (float)(ce_scale * (double)ir / NC);
-    }
-    for (int a = 0; a < NC; ++a) {
-        const int node = s_node[le][a];
-        const PB<D, T> b = pbasis<D, T>(a, q, inv_h);
-        for (int gf = 0; gf < NF; ++gf) {
-            // unit tangent in field gf at corner a (averages move by 1/2, differences by 1)
-            QPIn<D, Dual<T>> XD;
-            const T hf = T(0.5);
-            for (int i = 0; i < D; ++i) {
-                XD.v[i] = Dual<T>(X.v[i], gf == i ? hf * b.N : T(0));
-                for (int k = 0; k < D; ++k) XD.gv[i][k] = Dual<T>(X.gv[i][k], gf == i ? hf * b.dN[k] : T(0));
-                XD.vdt[i] = Dual<T>(X.vdt[i], gf == i ? inv_dt * b.N : T(0));
-                XD.gp[i] = Dual<T>(X.gp[i], gf == D ? hf * b.dN[i] : T(0));
-                XD.gphi[i] = Dual<T>(X.gphi[i], gf == D + 1 ? hf * b.dN[i] : T(0));
-                XD.gmu[i] = Dual<T>(X.gmu[i], gf == D + 2 ? hf * b.dN[i] : T(0));
-                const T pst = (gf == D + 1 && s_mask[le][a]) ? hf * b.dN[i] : T(0);
-                XD.gps[i] = Dual<T>(X.gps[i], pst);
-            }
-            XD.p = Dual<T>(X.p, gf == D ? hf * b.N : T(0));
-            XD.phi = Dual<T>(X.phi, gf == D + 1 ? hf * b.N : T(0));
-            XD.mu = Dual<T>(X.mu, gf == D + 2 ? hf * b.N : T(0));
-            for (int k = 0; k < NH; ++k) XD.H[k] = Dual<T>(X.H[k], gf == D + 1 ? hf * b.d2N[k] : T(0));
-            XD.phidt = Dual<T>(X.phidt, gf == D + 1 ? inv_dt * b.N : T(0));
-            T dv = T(0);
-            if (gf < D) dv = b.dN[gf];
-            XD.divnew = Dual<T>(X.divnew, dv);
-            XD.ps = Dual<T>(X.ps, (gf == D + 1 && s_mask[le][a]) ? hf * b.N : T(0));
-            QPOut<D, Dual<T>> F;
-            pointwise<D, Dual<T>, T>(XD, c, g, F);
-            for (int f = 0; f < NF; ++f) {
-                T v = b.N * F.f0[f].d;
-                for (int k = 0; k < D; ++k) v += b.dN[k] * F.f1[f][k].d;
-                v *= detJ;
-                for (int off = NC / 2; off > 0; off >>= 1) v += __shfl_xor_sync(lanes, v, off);
-                if (q == 0 && node >= 0) atomicAdd(blk + ((size_t)node * NF + f) * NF + gf, v);
-            }
-        }
-    }
 }
 
 // Replace Dirichlet / pin rows by identity rows and invert every block (Gauss-Jordan
@@ -711,29 +567,6 @@ __global__ void jacobi_kernel(const double* __restrict__ d, const double* __rest
     if (n < N) z[n] = r[n] / d[n];
 }
 
-template <class R>
-PCst<R> pcst_from(const PhysConst& pc) {
-    PCst<R> c;
-    c.alpha = R(pc.alpha);
-    c.beta = R(pc.beta);
-    c.gamma = R(pc.gamma);
-    c.xi = R(pc.xi);
-    c.Jc = R((pc.rho_minus - pc.rho_plus) / (2.0 * pc.rho_plus * pc.Cn));
-    c.inv_Pe = R(pc.inv_Pe);
-    c.inv_We = R(pc.inv_We);
-    c.inv_Re = R(pc.inv_Re);
-    c.inv_Fr = R(pc.inv_Fr);
-    c.Cn_We = R(pc.Cn * pc.inv_We);
-    c.inv_PeCn = R(1.0 / (pc.Pe * pc.Cn));
-    c.Cn2 = R(pc.Cn * pc.Cn);
-    c.Pe = R(pc.Pe);
-    c.Re = R(pc.Re);
-    c.four_over_dt2 = R(pc.four_over_dt2);
-    c.C_I = R(pc.C_I);
-    c.C_phi = R(pc.C_phi);
-    return c;
-}
-
 struct Ctx {
     chns_mesh* m;
     SolverWS* ws;
@@ -753,17 +586,6 @@ chns_status read_sc(Ctx& c, const double* dev, int k, double* host) {
 chns_status dot_host(Ctx& c, const double* a, const double* b, double* out) {
     CHNS_CUDA(launch_dot(c.m, a, b, c.n, c.ws->sc, c.s));
     return read_sc(c, c.ws->sc, 1, out);
-}
-
-template <int D, class T>
-cudaError_t pc_build_launch(const chns_mesh* m, const PhysConst& pc, const T* Uo, const T* Un, T* blk,
-                            float* ce, cudaStream_t s) {
-    constexpr int NC = 1 << D, EPB = 128 / NC;
-    cudaError_t e = cudaMemsetAsync(blk, 0, (size_t)m->dm.N * m->dm.nf * m->dm.nf * sizeof(T), s);
-    if (e != cudaSuccess) return e;
-    const double ce_scale = pc.dt / (2.0 * pc.We);
-    { pc_build_kernel<D, T><<<(unsigned)((m->dm.E + EPB - 1) / EPB), 128, 0, s>>>(m->dm, pcst_from<T>(pc), T(pc.inv_dt), Uo, Un, blk, ce, ce_scale); chns_count_launches(1); }
-    return cudaGetLastError();
 }
 
 // nodal psi''(phi~) with phi~ the mid-point average (FP32)
@@ -871,14 +693,10 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
         CHNS_CUDA(cudaEventRecord(ws->ev[2], c.s));
         if (mixed) {
             { to32_kernel<<<c.g, 256, 0, c.s>>>(U, ws->Us32, c.n); chns_count_launches(1); }
-            cudaError_t e = (D == 2) ? pc_build_launch<2, float>(m, pc, ws->Uo32, ws->Us32, ws->Pblk32, ws->ce, c.s)
-                                     : pc_build_launch<3, float>(m, pc, ws->Uo32, ws->Us32, ws->Pblk32, ws->ce, c.s);
-            CHNS_CUDA(e);
+            CHNS_CUDA(launch_pc_build(m, pc, ws->Uo32, ws->Us32, ws->Pblk32, ws->ce, c.s));
             { pc_invert_kernel<float, float><<<gN, 128, 0, c.s>>>(m->dm, ws->Pblk32, ws->Pinv32, pin, ws->S, ws->Sd, pcmask); chns_count_launches(1); }
         } else {
-            cudaError_t e = (D == 2) ? pc_build_launch<2, double>(m, pc, U_old, U, ws->Pblk64, ws->ce, c.s)
-                                     : pc_build_launch<3, double>(m, pc, U_old, U, ws->Pblk64, ws->ce, c.s);
-            CHNS_CUDA(e);
+            CHNS_CUDA(launch_pc_build(m, pc, U_old, U, ws->Pblk64, ws->ce, c.s));
             { pc_invert_kernel<double, double><<<gN, 128, 0, c.s>>>(m->dm, ws->Pblk64, ws->Pinv64, pin, ws->S, ws->Sd, pcmask); chns_count_launches(1); }
         }
         CHNS_CUDA(cudaGetLastError());
@@ -1334,9 +1152,7 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
     std::memset(&S, 0, sizeof(S));
 
     // nodal blocks of J (FP64) at the converged state; J^T's blocks are their transposes
-    cudaError_t ce = (D == 2) ? pc_build_launch<2, double>(m, pc, U_old, U_new, ws->Pblk64, ws->ce, c.s)
-                              : pc_build_launch<3, double>(m, pc, U_old, U_new, ws->Pblk64, ws->ce, c.s);
-    CHNS_CUDA(ce);
+    CHNS_CUDA(launch_pc_build(m, pc, U_old, U_new, ws->Pblk64, ws->ce, c.s));
     { pc_invert_kernel<double, double><<<gN, 128, 0, c.s>>>(m->dm, ws->Pblk64, ws->Pinv64, pin, ws->S, ws->Sd, schur ? 1 : 0); chns_count_launches(1); }
     if (schur) {
         if ((st = precond_setup(m, spec, ws->ce, nullptr, c.s)) != CHNS_OK) return st;

@@ -74,3 +74,26 @@ def test_not_finite_coefficients_are_reported(chns):
         with pytest.raises(chns.ChnsError) as e:
             chns.newton_step(gm, prm, chns.SolverOpts.make(precision=1, pc_type=pc, pc_degree=4), U0)
         assert e.value.name == "CHNS_ENAN" and "bound" in str(e.value)
+
+
+@pytest.mark.parametrize("dim,level,hi", [(2, 1, 1.0), (2, 4, 0.8), (3, 1, 1.0), (3, 3, 1.5)])
+def test_nodal_blocks_give_the_diagonal_of_the_jacobian(chns, dim, level, hi):
+    """Without hanging points the nodal blocks are exact, and the first norm a step reports is
+    ||R / |diag J|| with J's identity rows: both from the oracle.  FP64 blocks: 1e-11 (1e3
+    roundings over the quotient of two sums); FP32 blocks: 1e-4 (the same count at 6e-8)."""
+    from oracle import Mesh as OMesh, Oracle, Params as OParams
+    leaves = synth.uniform_leaves(dim, level)
+    om, gm = OMesh(dim, level, leaves, 0.0, hi), chns.Mesh(dim, level, leaves, 0.0, hi)
+    cfg = synth.config_params("drop3d" if dim == 3 else "drop2d")
+    cfg.update(Fr=1.0, rho_ratio=20.0, eta_ratio=7.0, Cn=0.05)
+    prm, oprm, o = chns.Params.make(**cfg), OParams(**cfg), Oracle(om)
+    rng = np.random.default_rng(11)
+    U = 0.1 * rng.standard_normal((om.N, dim + 3))
+    U[:, dim + 1] = 1.2 * np.sin(4.0 * om.x.sum(axis=1))
+    Ut = torch.tensor(U)
+    dg = np.abs(np.asarray(o.jacobian(oprm, Ut, Ut).diagonal())).reshape(U.shape)
+    want = float(np.linalg.norm(o.residual(oprm, Ut, Ut).numpy() / dg))
+    for prec, tol in ((0, 1e-11), (1, 1e-4)):
+        opts = chns.SolverOpts.make(precision=prec, pc_type=0, max_newton=0)
+        _, st = chns.newton_step(gm, prm, opts, Ut.cuda(), check=False)
+        assert abs(st.res0 - want) <= tol * want, (prec, st.res0, want)
