@@ -1,0 +1,276 @@
+// Vector kernels of the Arnoldi process (Newton's GMRES and the adjoint's), FP64.
+//
+// The basis is kept unnormalised: slot j of V holds w_j and a device scalar s_j = 1/|w_j|, and
+// v_j = s_j w_j.  The scale rides along where a vector is read anyway, so no pass normalises.
+// One Gram-Schmidt pass is a dot kernel (32 columns at a time, forming w = S y + mean on the way)
+// and an update kernel with the new norm; the last block of each sums the partials, in a fixed
+// order, and the update's writes what the host waits for into pinned memory.  A second pass is
+// queued behind the first and decided on the device: its blocks return at once when |w| kept a
+// tenth of its length.  (Left to the host, it costs a discarded operator application whenever it
+// is wanted, which is often: two drops, 81 -> 118 ms per Newton step.)
+//
+// Bound: k FP64 FMAs per entry and pass on the narrow FP64 pipe (n = 1.65 M, k = 15: 39 us) next
+// to one read of V (29 us).  The kernels are instantiated per number of columns (dots) or per
+// remainder (update), so that all loads of an entry pair go out together, and few threads take many
+// rows, so that the reductions add 5 % of FP64 work instead of the 60 % of eight columns per
+// thread.  The update walks the rows backwards, where the dot pass has just left its columns in L2
+// (evict-first loads there: 34 -> 50 us).
+//   n = 1.65 M, k = 1..30: dots 3.3 us per column + 24 us (w formed, 4 us of reduction), update
+//   2.7 us per column + 10 us; all of an Arnoldi step's vector work 181 -> 136 us, and without the
+//   33 us of the normalising, scaling and mean passes that it takes in.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "chns_internal.h"
+#include "krylov.h"
+
+namespace krylov {
+
+namespace {
+
+__device__ __forceinline__ double formed(const Source& s, int64_t i, double mean) {
+    const double y = s.yf ? (double)s.yf[i] : s.yd[i];
+    const double w = s.S[i] * y;
+    return s.mean && (int)((uint32_t)i % (uint32_t)s.NF) == s.f ? w + mean : w;   // n < 2^32
+}
+
+// h = s .* (V^T w) for K <= 32 columns starting at V, and |w|^2 (nrm not null).  With a source w is
+// formed here and slot w gets it.  pred: return unless it is 1.
+template <int K>
+__global__ void __launch_bounds__(T, 2)
+dots_kernel(const double* __restrict__ V, int64_t ld, Source src, double* w, int64_t n, const double* __restrict__ scale,
+            double* __restrict__ h, double* __restrict__ nrm, double* __restrict__ partials, unsigned int* counter,
+            const double* __restrict__ pred) {
+    if (pred && pred[0] == 0.0) return;
+    constexpr int KP = K <= 1 ? 1 : K <= 2 ? 2 : K <= 4 ? 4 : K <= 8 ? 8 : K <= 16 ? 16 : 32;   // halves evenly
+    double acc[KP], nn = 0.0;
+#pragma unroll
+    for (int j = 0; j < KP; ++j) acc[j] = 0.0;
+    const bool form = src.yf || src.yd;
+    const double mean = src.mean ? src.a * src.mean[0] : 0.0;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x * 2, full_pairs = n / 2 * 2;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 2; i < full_pairs; i += stride) {
+        double2 x;
+        if (form) {
+            x = make_double2(formed(src, i, mean), formed(src, i + 1, mean));
+            *reinterpret_cast<double2*>(w + i) = x;
+        } else {
+            x = *reinterpret_cast<const double2*>(w + i);
+        }
+        const double* p = V + i;
+        // the columns' loads are independent: as many in flight as the registers hold
+        double2 v[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) v[j] = *reinterpret_cast<const double2*>(p + (size_t)j * ld);
+        if (nrm) nn = fma(x.y, x.y, fma(x.x, x.x, nn));
+#pragma unroll
+        for (int j = 0; j < K; ++j) acc[j] = fma(v[j].y, x.y, fma(v[j].x, x.x, acc[j]));
+    }
+    if (full_pairs < n && blockIdx.x == 0 && threadIdx.x == 0) {
+        const int64_t i = n - 1;
+        const double x = form ? formed(src, i, mean) : w[i];
+        if (form) w[i] = x;
+        nn = fma(x, x, nn);
+#pragma unroll
+        for (int j = 0; j < K; ++j) acc[j] = fma(V[(size_t)j * ld + i], x, acc[j]);
+    }
+    // halve the numbers over the warp's lanes, then one number per lane group
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int base = 0, cnt = KP;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        if (cnt > 1) {
+            cnt /= 2;
+            const bool up = lane & o;
+#pragma unroll
+            for (int t = 0; t < KP / 2; ++t) {
+                if (t >= cnt) break;
+                const double keep = up ? acc[cnt + t] : acc[t], give = up ? acc[t] : acc[cnt + t];
+                acc[t] = keep + __shfl_xor_sync(full, give, o);
+            }
+            base += up ? cnt : 0;
+        } else {
+            acc[0] += __shfl_xor_sync(full, acc[0], o);
+        }
+    }
+    __shared__ double sh[T / 32][KP + 1];
+    __shared__ double fin[T];
+    sh[warp][base] = acc[0];   // lanes that share a number hold the same sum
+    if (nrm) {
+        nn = warp_sum(nn);
+        if (lane == 0) sh[warp][KP] = nn;
+    }
+    __syncthreads();
+    if (threadIdx.x <= KP && (threadIdx.x < KP || nrm)) {
+        double v = 0.0;
+        for (int q = 0; q < (int)blockDim.x / 32; ++q) v += sh[q][threadIdx.x];
+        partials[(size_t)blockIdx.x * (KP + 1) + threadIdx.x] = v;
+    }
+    if (!last_block(counter)) return;
+    // thread (g, j) adds up number j of blocks g, g + groups, ...: eight loads in flight, so that this
+    // tail is a few memory latencies long
+    const int groups = blockDim.x / KP, g = threadIdx.x / KP, num = threadIdx.x % KP;
+    double v = 0.0;
+#pragma unroll 8
+    for (int b = g; b < (int)gridDim.x; b += groups) v += __ldcg(partials + (size_t)b * (KP + 1) + num);
+    fin[threadIdx.x] = v;
+    if (nrm) {
+        double t = 0.0;
+#pragma unroll 4
+        for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) t += __ldcg(partials + (size_t)b * (KP + 1) + KP);
+        t = warp_sum(t);
+        if (lane == 0) sh[warp][KP] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < K) {
+        double t = 0.0;
+#pragma unroll 8
+        for (int q = 0; q < groups; ++q) t += fin[q * KP + threadIdx.x];
+        h[threadIdx.x] = t * scale[threadIdx.x];
+    }
+    if (nrm && threadIdx.x == blockDim.x - 1) {
+        double t = 0.0;
+        for (int q = 0; q < (int)blockDim.x / 32; ++q) t += sh[q][KP];
+        nrm[0] = t;
+    }
+}
+
+// w -= sum_j h_j v_j over k = 8 a + REM columns (the remainder's loads go out together as well),
+// and |w|^2 of the result.  The last block keeps the books: FIRST decides whether |w|^2 fell below
+// thr times its old value (then a second pass follows); s_next = 1/|w| (0 on breakdown, which the
+// host reports); host (pinned) gets the coefficients of both passes together and the norm.
+template <int J>
+__device__ __forceinline__ void update_columns(const double* __restrict__ p, int64_t ld, const double* c, double2& s) {
+    double2 v[J > 0 ? J : 1];
+#pragma unroll
+    for (int j = 0; j < J; ++j) v[j] = *reinterpret_cast<const double2*>(p + (size_t)j * ld);
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        s.x = fma(c[j], v[j].x, s.x);
+        s.y = fma(c[j], v[j].y, s.y);
+    }
+}
+template <bool FIRST, int REM>
+__global__ void __launch_bounds__(T, 4) update_kernel(const double* __restrict__ V, int64_t ld, int k, double* w, int64_t n,
+                                                      double* __restrict__ sc, double* __restrict__ s_next, double thr,
+                                                      double* host, double* __restrict__ partials, unsigned int* counter) {
+    if (!FIRST && sc[SC_AGAIN] == 0.0) return;
+    extern __shared__ double c[];   // k coefficients
+    const double* h = sc + (FIRST ? SC_H1 : SC_H2);
+    for (int j = threadIdx.x; j < k; j += blockDim.x) c[j] = -h[j] * sc[SC_SCALE + j];
+    __syncthreads();
+    double nn = 0.0;
+    const int64_t pairs = (n + 1) / 2, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < pairs; q += stride) {
+        const int64_t i = (pairs - 1 - q) * 2;
+        const double* p = V + i;
+        double2 s;
+        if (i + 1 < n) {
+            s = *reinterpret_cast<const double2*>(w + i);
+            int j = 0;
+            for (; j + 8 <= k; j += 8) update_columns<8>(p + (size_t)j * ld, ld, c + j, s);
+            update_columns<REM>(p + (size_t)j * ld, ld, c + j, s);
+            *reinterpret_cast<double2*>(w + i) = s;
+        } else {
+            s = make_double2(w[i], 0.0);
+            for (int j = 0; j < k; ++j) s.x = fma(c[j], p[(size_t)j * ld], s.x);
+            w[i] = s.x;
+        }
+        nn = fma(s.y, s.y, fma(s.x, s.x, nn));
+    }
+    __shared__ double sh[T / 32];
+    nn = warp_sum(nn);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = nn;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = 0.0;
+        for (int q = 0; q < (int)blockDim.x / 32; ++q) v += sh[q];
+        partials[blockIdx.x] = v;
+    }
+    if (!last_block(counter)) return;
+    double v = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) v += __ldcg(partials + b);
+    v = warp_sum(v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double tot = 0.0;
+    for (int q = 0; q < (int)blockDim.x / 32; ++q) tot += sh[q];
+    for (int j = threadIdx.x; j < k; j += blockDim.x) host[j] = FIRST ? sc[SC_H1 + j] : sc[SC_H1 + j] + sc[SC_H2 + j];
+    if (threadIdx.x == 0) {
+        if (FIRST) sc[SC_AGAIN] = tot < thr * sc[SC_NB] ? 1.0 : 0.0;
+        host[SC_NA] = tot;
+        s_next[0] = tot > 0.0 ? 1.0 / sqrt(tot) : 0.0;
+    }
+    __threadfence_system();
+}
+
+// u = sum_{j<k} y_j v_j
+__global__ void combine_kernel(const double* __restrict__ V, int64_t ld, int k, const double* __restrict__ y,
+                               const double* __restrict__ scale, double* __restrict__ u, int64_t n) {
+    extern __shared__ double c[];
+    for (int j = threadIdx.x; j < k; j += blockDim.x) c[j] = y[j] * scale[j];
+    __syncthreads();
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        double s = 0.0;
+#pragma unroll 4
+        for (int j = 0; j < k; ++j) s = fma(c[j], V[(size_t)j * ld + i], s);
+        u[i] = s;
+    }
+}
+
+template <bool FIRST>
+void launch_update(int nu, int th, const double* V, int64_t ld, int k, double* w, int64_t n, double* sc, double* sk, double thr,
+                   double* host, double* partials, unsigned int* counter, cudaStream_t st) {
+    const size_t sh = k * sizeof(double);
+    switch (k % 8) {
+#define CHNS_UPDATE(R) case R: update_kernel<FIRST, R><<<nu, th, sh, st>>>(V, ld, k, w, n, sc, sk, thr, host, partials, counter); break
+        CHNS_UPDATE(0); CHNS_UPDATE(1); CHNS_UPDATE(2); CHNS_UPDATE(3);
+        CHNS_UPDATE(4); CHNS_UPDATE(5); CHNS_UPDATE(6); CHNS_UPDATE(7);
+#undef CHNS_UPDATE
+    }
+}
+template <int K = 32>
+void launch_dots(int kk, int nb, int th, const double* V, int64_t ld, const Source& s, double* w, int64_t n, const double* scale,
+                 double* h, double* nrm, double* partials, unsigned int* counter, const double* pred, cudaStream_t st) {
+    if (kk == K) dots_kernel<K><<<nb, th, 0, st>>>(V, ld, s, w, n, scale, h, nrm, partials, counter, pred);
+    else if constexpr (K > 1) launch_dots<K - 1>(kk, nb, th, V, ld, s, w, n, scale, h, nrm, partials, counter, pred, st);
+}
+}  // namespace
+
+int orthogonalise(double* V, int64_t ld, int k, const Source& src, int64_t n, double* sc, double thr, double* host, double* partials,
+                  unsigned int* counter, cudaStream_t st) {
+    // small vectors take two-warp blocks: the reductions are FP64 work per block, and the FP64 pipe
+    // is per SM
+    const int64_t sms = chns_num_sms();
+    const int th = n < 256 * sms ? 64 : T;
+    const int64_t need = (n + 2 * th - 1) / (2 * th);
+    const int nb = (int)std::min<int64_t>(need, 2 * (T / th) * sms);
+    const int nu = (int)std::min<int64_t>(need, 4 * (T / th) * sms);
+    double* w = V + (size_t)k * ld;
+    int nk = 0;
+    for (bool first : {true, false}) {
+        for (int j0 = 0; j0 < k; j0 += 32) {
+            Source s = src;
+            const bool form = first && j0 == 0;
+            if (!form) s.yf = nullptr, s.yd = nullptr, s.mean = nullptr;
+            launch_dots(std::min(k - j0, 32), nb, th, V + (size_t)j0 * ld, ld, s, w, n, sc + SC_SCALE + j0,
+                        sc + (first ? SC_H1 : SC_H2) + j0, form ? sc + SC_NB : nullptr, partials, counter,
+                        first ? nullptr : sc + SC_AGAIN, st);
+            ++nk;
+        }
+        double* sk = sc + SC_SCALE + k;
+        if (first) launch_update<true>(nu, th, V, ld, k, w, n, sc, sk, thr, host, partials, counter, st);
+        else launch_update<false>(nu, th, V, ld, k, w, n, sc, sk, thr, host, partials, counter, st);
+        ++nk;
+    }
+    return nk;
+}
+void combine(const double* V, int64_t ld, int k, const double* y, const double* scale, double* u, int64_t n, cudaStream_t st) {
+    const int64_t need = (n + T - 1) / T, cap = 8 * (int64_t)chns_num_sms();
+    combine_kernel<<<(unsigned)std::min(need, cap), T, k * sizeof(double), st>>>(V, ld, k, y, scale, u, n);
+}
+
+}  // namespace krylov

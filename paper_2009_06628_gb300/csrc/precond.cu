@@ -386,63 +386,72 @@ __device__ __forceinline__ int64_t my_row(int64_t N, bool& store) {
     return r < N ? r : N - 1;
 }
 
-// r = v_f (strided FP64 field) and d = dinv r / theta
-__global__ void cheb_init_kernel(int64_t N, int NF, int f, const double* __restrict__ v, const float* __restrict__ dinv,
-                                 const ChebCoef* __restrict__ cf, float* __restrict__ r, float* __restrict__ d) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    const float rv = (float)v[(size_t)n * NF + f];
-    r[n] = rv;
-    d[n] = cf->inv_theta * dinv[n] * rv;
+// Adds m_n z_n of a block's threads to its partial; the block that finishes last sums the
+// partials in a fixed order.  All threads of the block call it.
+__device__ __forceinline__ void mean_add(const PrecondMean& M, double v) {
+    // one warp adds up the block's values (13 FP64 instructions; a shuffle tree in every warp is 40
+    // on a pipe that takes one per 16 cycles)
+    __shared__ double sh[256];
+    __shared__ bool last;
+    const int lane = threadIdx.x;
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    if (lane < 32) {
+        v = 0.0;
+        for (int q = lane; q < (int)blockDim.x; q += 32) v += sh[q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) {
+            M.partials[blockIdx.x] = v;
+            __threadfence();
+            last = atomicAdd(M.counter, 1u) == gridDim.x - 1;
+            if (last) *M.counter = 0u;
+        }
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    v = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) v += __ldcg(M.partials + b);
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    if (lane < 32) {
+        v = 0.0;
+        for (int q = lane; q < (int)blockDim.x; q += 32) v += sh[q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) M.out[0] = v;
+    }
 }
-// Chebyshev step k: r -= A d; d' = c1 d + c2 dinv r; x (+)= d (k = 0 writes x).  LAST: the
-// result base + x + d + d' goes to z (strided field f; z may be base) and r, d' are not kept.
-template <int LPR, bool LAST, class TO>
+
+// Chebyshev step k: r -= A d; d' = c1 d + c2 dinv r; x (+)= d.  FIRST: r is the right-hand side b
+// and d = dinv b / theta is formed where it is gathered, x = 0.  LAST: the result base + x + d + d'
+// goes to z (strided field f; z may be base, base may be null) and r, d' are not kept.
+template <int LPR, bool FIRST, bool LAST, class TO>
 __global__ void __launch_bounds__(256) cheb_step_kernel(Sell S, const float* __restrict__ val,
                                                         const float* __restrict__ dinv,
                                                         const ChebCoef* __restrict__ cf, int k,
-                                                        const float* __restrict__ d, float* __restrict__ dn,
-                                                        float* __restrict__ r, float* __restrict__ x,
-                                                        const float* base, TO* z, int NF, int f) {
+                                                        const float* __restrict__ b, const float* __restrict__ d,
+                                                        float* __restrict__ dn, float* __restrict__ r,
+                                                        float* __restrict__ x, const float* base, TO* z, int NF, int f,
+                                                        PrecondMean mean) {
     bool store;
     const int64_t n = my_row<LPR>(S.N, store);
-    const float dd = d[n], rr = r[n], di = dinv[n], xx = k == 0 ? 0.0f : x[n];
-    const float rn = rr - row_dot<LPR>(S, val, n, [&](int q) { return __ldg(d + q); });
-    const float dv = cf->c1[k] * dd + cf->c2[k] * di * rn;
-    if (!store) return;
+    const float di = dinv[n], it = FIRST ? cf->inv_theta : 0.0f;
+    const float rr = FIRST ? b[n] : r[n], dd = FIRST ? it * di * rr : d[n], xx = FIRST ? 0.0f : x[n];
+    float y;
+    if (FIRST) y = row_dot<LPR>(S, val, n, [&](int q) { return it * __ldg(dinv + q) * __ldg(b + q); });
+    else y = row_dot<LPR>(S, val, n, [&](int q) { return __ldg(d + q); });
+    const float rn = rr - y, dv = cf->c1[k] * dd + cf->c2[k] * di * rn;
     if (LAST) {
-        const float v = (xx + dd) + dv;
-        z[(size_t)n * NF + f] = (TO)(base ? base[n] + v : v);
-    } else {
+        const float v = base ? base[n] + ((xx + dd) + dv) : (xx + dd) + dv;
+        if (store) z[(size_t)n * NF + f] = (TO)v;
+        if (mean.out) mean_add(mean, store ? mean.nmass[n] * (double)v : 0.0);
+    } else if (store) {
         x[n] = xx + dd;
         r[n] = rn;
         dn[n] = dv;
     }
-}
-__global__ void load_kernel(int64_t N, int NF, int f, const double* __restrict__ v, float* __restrict__ b) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) b[n] = (float)v[(size_t)n * NF + f];
-}
-__global__ void cheb_start_kernel(int64_t N, const float* __restrict__ b, const float* __restrict__ dinv,
-                                  const ChebCoef* __restrict__ cf, float* __restrict__ r, float* __restrict__ d) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    r[n] = b[n];
-    d[n] = cf->inv_theta * dinv[n] * b[n];
-}
-// degree-2 smoother in one pass (d_0 = dinv b / theta is formed where it is gathered):
-// z = base + d_0 + (c1 d_0 + c2 dinv (b - A d_0)); base may be null, or z
-template <int LPR, class TO>
-__global__ void __launch_bounds__(256) cheb2_kernel(Sell S, const float* __restrict__ val, const float* __restrict__ dinv,
-                                                    const ChebCoef* __restrict__ cf, const float* __restrict__ b,
-                                                    const float* base, TO* z, int NF, int f) {
-    bool store;
-    const int64_t n = my_row<LPR>(S.N, store);
-    const float it = cf->inv_theta, bn = b[n], di = dinv[n], d0 = it * di * bn;
-    const float y = row_dot<LPR>(S, val, n, [&](int q) { return it * __ldg(dinv + q) * __ldg(b + q); });
-    if (!store) return;
-    const float v = d0 + (cf->c1[0] * d0 + cf->c2[0] * di * (bn - y));
-    z[(size_t)n * NF + f] = (TO)(base ? base[n] + v : v);
 }
 // t = b - A x (t may be b)
 template <int LPR>
@@ -454,45 +463,35 @@ __global__ void __launch_bounds__(256) residual_kernel(Sell S, const float* __re
     if (store) t[n] = b[n] - y;
 }
 template <class TO>
-__global__ void store_kernel(int64_t N, int NF, int f, const float* __restrict__ x, TO* __restrict__ z) {
+__global__ void store_kernel(int64_t N, int NF, int f, const float* __restrict__ x, TO* __restrict__ z, PrecondMean mean) {
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) z[(size_t)n * NF + f] = (TO)x[n];
+    const float v = n < N ? x[n] : 0.0f;
+    if (n < N) z[(size_t)n * NF + f] = (TO)v;
+    if (mean.out) mean_add(mean, n < N ? mean.nmass[n] * (double)v : 0.0);
 }
-// Cahn-Hilliard block.  rm = v_mu, a = rm / ml, rp = v_phi
-__global__ void ch_load_kernel(int64_t N, int NF, int fphi, const double* __restrict__ v, const float* __restrict__ ml,
-                               float* __restrict__ rp, float* __restrict__ rm, float* __restrict__ a) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    rp[n] = (float)v[(size_t)n * NF + fphi];
-    const float t = (float)v[(size_t)n * NF + fphi + 1];
-    rm[n] = t;
-    a[n] = t / ml[n];
-}
-// r = base + c A x, d = dinv r / theta: the right-hand side of a Chebyshev solve
+// r = base + c A (x .* m): the right-hand side of a Chebyshev solve (base, m may be null)
 template <int LPR>
 __global__ void __launch_bounds__(256) rhs_kernel(Sell S, const float* __restrict__ val, const float* __restrict__ x,
-                                                  const float* __restrict__ base, float c,
-                                                  const float* __restrict__ dinv, const ChebCoef* __restrict__ cf,
-                                                  float* __restrict__ r, float* __restrict__ d) {
+                                                  const float* __restrict__ m, const float* __restrict__ base, float c,
+                                                  float* __restrict__ r) {
     bool store;
     const int64_t n = my_row<LPR>(S.N, store);
-    const float y = row_dot<LPR>(S, val, n, [&](int q) { return __ldg(x + q); });
-    if (!store) return;
-    const float rv = base ? base[n] + c * y : c * y;
-    r[n] = rv;
-    d[n] = cf->inv_theta * dinv[n] * rv;
+    float y;
+    if (m) y = row_dot<LPR>(S, val, n, [&](int q) { return __ldg(m + q) * __ldg(x + q); });
+    else y = row_dot<LPR>(S, val, n, [&](int q) { return __ldg(x + q); });
+    if (store) r[n] = base ? base[n] + c * y : c * y;
 }
-// z_phi = x, z_mu = psi2 x + Cn^2 (K x) / ml - 2 rm / ml
+// Cahn-Hilliard block, last pass: z_phi = x, z_mu = psi2 x + (Cn^2 K x - 2 r_mu) / m_l (lumped mass)
 template <int LPR, class TO>
 __global__ void __launch_bounds__(256) ch_store_kernel(Sell S, const float* __restrict__ vk, int NF, int fphi,
                                                        const float* __restrict__ x, const float* __restrict__ rm,
-                                                       const float* __restrict__ psi2, const float* __restrict__ ml,
+                                                       const float* __restrict__ psi2, const float* __restrict__ iml,
                                                        float cn2, TO* __restrict__ z) {
     bool store;
     const int64_t n = my_row<LPR>(S.N, store);
     const float kx = row_dot<LPR>(S, vk, n, [&](int q) { return __ldg(x + q); });
     if (!store) return;
-    const float xv = x[n], il = 1.0f / ml[n];
+    const float xv = x[n], il = iml[n];
     z[(size_t)n * NF + fphi] = (TO)xv;
     z[(size_t)n * NF + fphi + 1] = (TO)(psi2[n] * xv + cn2 * kx * il - 2.0f * rm[n] * il);
 }
@@ -505,9 +504,9 @@ __global__ void restrict_ce_kernel(int64_t Ef, int D, const int32_t* __restrict_
     const int c = fmap[e];
     atomicAdd(ce_c + c, ldexpf(ce_f[e], -D * ((int)lev_f[e] - (int)lev_c[c])));
 }
-__global__ void ml_kernel(int64_t N, const double* __restrict__ nmass, float* __restrict__ ml) {
+__global__ void iml_kernel(int64_t N, const double* __restrict__ nmass, float* __restrict__ iml) {
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) ml[n] = (float)nmass[n];
+    if (n < N) iml[n] = 1.0f / (float)nmass[n];
 }
 
 // ---------------- small levels: one block ----------------
@@ -585,7 +584,7 @@ __device__ void tail_cheb(const TailLevel& L, const float* in, float* out) {
     if (L.S.N * 8 <= TAIL_THREADS) tail_cheb_l<8, ADD>(L, in, out);
     else tail_cheb_l<1, ADD>(L, in, out);
 }
-// V-cycle over the block's levels: L[0].b -> L[0].x
+// V-cycle over the block's levels (one level: its polynomial): L[0].b -> L[0].x
 __global__ void __launch_bounds__(TAIL_THREADS) tail_kernel(const Tail* __restrict__ tp) {
     const Tail& T = *tp;
     const int64_t t0 = threadIdx.x, nt = TAIL_THREADS;
@@ -612,17 +611,6 @@ __global__ void __launch_bounds__(TAIL_THREADS) tail_kernel(const Tail* __restri
         tail_cheb<true>(L, L.b, L.x);
     }
 }
-// The whole polynomial of a small mesh: v_f (strided) -> z_f.
-template <class TO>
-__global__ void __launch_bounds__(TAIL_THREADS) tail_cheb_kernel(const Tail* __restrict__ tp, const double* __restrict__ v,
-                                                                 TO* __restrict__ z, int NF, int f) {
-    const TailLevel& L = tp->L[0];
-    for (int64_t n = threadIdx.x; n < L.S.N; n += TAIL_THREADS) L.b[n] = (float)v[(size_t)n * NF + f];
-    __syncthreads();
-    tail_cheb<false>(L, L.b, L.x);
-    for (int64_t n = threadIdx.x; n < L.S.N; n += TAIL_THREADS) z[(size_t)n * NF + f] = (TO)L.x[n];
-}
-
 template <class T>
 cudaError_t alloc(T** p, int64_t n) {
     return *p ? cudaSuccess : cudaMalloc((void**)p, (size_t)std::max<int64_t>(n, 1) * sizeof(T));
@@ -670,8 +658,8 @@ struct PrecondWS {
     unsigned int* flags = nullptr;
     // Cahn-Hilliard block on the mesh
     Sell SC;
-    float *vm = nullptr, *vk = nullptr, *va = nullptr, *ch_dinv = nullptr, *ml = nullptr, *rm = nullptr, *rp = nullptr,
-          *ca = nullptr, *cr = nullptr, *cx = nullptr, *cd0 = nullptr, *cd1 = nullptr;
+    float *vm = nullptr, *vk = nullptr, *va = nullptr, *ch_dinv = nullptr, *iml = nullptr, *rm = nullptr, *rp = nullptr,
+          *cb = nullptr, *ca = nullptr, *cr = nullptr, *cx = nullptr, *cd0 = nullptr, *cd1 = nullptr;
     const float* psi2 = nullptr;
     Tail* tail = nullptr;        // device descriptor of the one-block kernel's levels
     int tail_from = -1, tail_deg = 0;
@@ -681,7 +669,7 @@ struct PrecondWS {
     bool no_graphs = false;
     struct Graph {
         cudaGraphExec_t exec = nullptr;
-        const void *v = nullptr, *z = nullptr;
+        const void *mean = nullptr, *z = nullptr;
         size_t to = 0;
         PrecondSpec spec;
         int nk = 0;
@@ -851,48 +839,45 @@ void launch_residual_rows(const Level& L, float* t, cudaStream_t st) {   // t = 
     });
 }
 
-// polynomial of degree deg with r, d0 set: result (plus base) to z
+// z = base + polynomial of b (b is not x); the pressure's mean with it where asked for
 template <class TO>
-int cheb_steps(const Sell& S, const float* val, const float* dinv, const ChebCoef* cf, int deg, float* r, float* x,
-               float* d0, float* d1, const float* base, TO* z, int NF, int f, cudaStream_t st) {
+int cheb(const Sell& S, const float* val, const float* dinv, const ChebCoef* cf, int deg, const float* b, float* r, float* x,
+         float* d0, float* d1, const float* base, TO* z, int NF, int f, const PrecondMean& mean, cudaStream_t st) {
     split(S.N, [&](auto lpr) {
         constexpr int LPR = decltype(lpr)::value;
         const int g = blocks_for(S.N * LPR);
         for (int k = 0; k + 1 < deg; ++k) {
-            if (k + 2 == deg) cheb_step_kernel<LPR, true, TO><<<g, 256, 0, st>>>(S, val, dinv, cf, k, d0, d1, r, x, base, z, NF, f);
-            else cheb_step_kernel<LPR, false, TO><<<g, 256, 0, st>>>(S, val, dinv, cf, k, d0, d1, r, x, nullptr, z, NF, f);
+            const bool last = k + 2 == deg;
+            auto run = [&](auto first, auto fin) {
+                cheb_step_kernel<LPR, decltype(first)::value, decltype(fin)::value, TO><<<g, 256, 0, st>>>(
+                    S, val, dinv, cf, k, b, d0, d1, r, x, base, z, NF, f, mean);
+            };
+            if (k == 0 && last) run(std::true_type(), std::true_type());
+            else if (k == 0) run(std::true_type(), std::false_type());
+            else if (last) run(std::false_type(), std::true_type());
+            else run(std::false_type(), std::false_type());
             std::swap(d0, d1);
         }
     });
     return deg - 1;
 }
-// z = base + polynomial of b on level l (b: not t)
+// z = base + polynomial of the level's b
 template <class TO>
-int smooth(const Level& L, const ChebCoef* cf, int deg, const float* b, const float* base, TO* z, int NF, int f,
+int smooth(const Level& L, const ChebCoef* cf, int deg, const float* base, TO* z, int NF, int f, const PrecondMean& mean,
            cudaStream_t st) {
-    const int g = blocks_for(L.dm.N);
-    if (deg == 2) {
-        split(L.dm.N, [&](auto lpr) {
-            constexpr int LPR = decltype(lpr)::value;
-            cheb2_kernel<LPR, TO><<<blocks_for(L.dm.N * LPR), 256, 0, st>>>(L.S, L.val, L.dinv, cf, b, base, z, NF, f);
-        });
-        return 1;
-    }
-    cheb_start_kernel<<<g, 256, 0, st>>>(L.dm.N, b, L.dinv, cf, L.r, L.d0);
-    return 1 + cheb_steps<TO>(L.S, L.val, L.dinv, cf, deg, L.r, L.t, L.d0, L.d1, base, z, NF, f, st);
+    return cheb<TO>(L.S, L.val, L.dinv, cf, deg, L.b, L.r, L.t, L.d0, L.d1, base, z, NF, f, mean, st);
 }
-// One V-cycle, b from field f of v, result to field f of z: on every level pre-smoothing from 0,
+// One V-cycle from level 0's b, result to field f of z: on every level pre-smoothing from 0,
 // residual, restriction, the coarser cycle, prolongation, residual (in place of b), post-smoothing.
 template <class TO>
-cudaError_t vcycle(chns_mesh* m, const PrecondSpec& spec, const double* v, TO* z, int NF, int f, cudaStream_t st, int* nk) {
+cudaError_t vcycle(chns_mesh* m, const PrecondSpec& spec, TO* z, int NF, int f, const PrecondMean& mean, cudaStream_t st,
+                   int* nk) {
     PrecondWS* p = m->pre;
     const int from = p->tail_from;
     Level& L0 = p->lv[0];
-    load_kernel<<<blocks_for(L0.dm.N), 256, 0, st>>>(L0.dm.N, NF, f, v, L0.b);
-    ++*nk;
     for (int l = 0; l < from; ++l) {
         Level& L = p->lv[(size_t)l];
-        *nk += smooth<float>(L, p->cf + l, spec.degree, L.b, nullptr, L.x, 1, 0, st);
+        *nk += smooth<float>(L, p->cf + l, spec.degree, nullptr, L.x, 1, 0, PrecondMean(), st);
         launch_residual_rows(L, L.t, st);
         const cudaError_t e = transfer_apply_f32(m->mg->lv[(size_t)l + 1].P, true, false, L.t, p->lv[(size_t)l + 1].b, st);
         if (e != cudaSuccess) return e;
@@ -906,55 +891,57 @@ cudaError_t vcycle(chns_mesh* m, const PrecondSpec& spec, const double* v, TO* z
         if (e != cudaSuccess) return e;
         launch_residual_rows(L, L.b, st);
         *nk += 2;
-        *nk += l == 0 ? smooth<TO>(L, p->cf, spec.degree, L.b, L.x, z, NF, f, st)
-                      : smooth<float>(L, p->cf + l, spec.degree, L.b, L.x, L.x, 1, 0, st);
+        *nk += l == 0 ? smooth<TO>(L, p->cf, spec.degree, L.x, z, NF, f, mean, st)
+                      : smooth<float>(L, p->cf + l, spec.degree, L.x, L.x, 1, 0, PrecondMean(), st);
     }
     if (from == 0) {
-        store_kernel<TO><<<blocks_for(L0.dm.N), 256, 0, st>>>(L0.dm.N, NF, f, L0.x, z);
+        store_kernel<TO><<<blocks_for(L0.dm.N), 256, 0, st>>>(L0.dm.N, NF, f, L0.x, z, mean);
         ++*nk;
     }
     return cudaGetLastError();
 }
 template <class TO>
-cudaError_t polynomial(chns_mesh* m, const PrecondSpec& spec, const double* v, TO* z, int NF, int f, cudaStream_t st, int* nk) {
+cudaError_t polynomial(chns_mesh* m, const PrecondSpec& spec, TO* z, int NF, int f, const PrecondMean& mean, cudaStream_t st,
+                       int* nk) {
     PrecondWS* p = m->pre;
     Level& L = p->lv[0];
     if (p->tail_from == 0) {
-        tail_cheb_kernel<TO><<<1, TAIL_THREADS, 0, st>>>(p->tail, v, z, NF, f);
-        ++*nk;
+        tail_kernel<<<1, TAIL_THREADS, 0, st>>>(p->tail);
+        store_kernel<TO><<<blocks_for(L.dm.N), 256, 0, st>>>(L.dm.N, NF, f, L.x, z, mean);
+        *nk += 2;
         return cudaGetLastError();
     }
-    cheb_init_kernel<<<blocks_for(L.dm.N), 256, 0, st>>>(L.dm.N, NF, f, v, L.dinv, p->cf, L.r, L.d0);
-    *nk += 1 + cheb_steps<TO>(L.S, L.val, L.dinv, p->cf, spec.degree, L.r, L.x, L.d0, L.d1, nullptr, z, NF, f, st);
+    *nk += smooth<TO>(L, p->cf, spec.degree, nullptr, z, NF, f, mean, st);
     return cudaGetLastError();
 }
 // phi and mu: mu eliminated with the lumped mass, the phi Schur complement by two polynomials
 template <class TO>
-cudaError_t cahn_hilliard(chns_mesh* m, const PrecondSpec& spec, const double* v, TO* z, int NF, int f, cudaStream_t st,
-                          int* nk) {
+cudaError_t cahn_hilliard(chns_mesh* m, const PrecondSpec& spec, TO* z, int NF, int f, cudaStream_t st, int* nk) {
     PrecondWS* p = m->pre;
     const int64_t N = m->dm.N;
-    const int g = blocks_for(N);
     const ChebCoef* cf = p->cf + TAIL_LEVELS;
-    ch_load_kernel<<<g, 256, 0, st>>>(N, NF, f, v, p->ml, p->rp, p->rm, p->ca);
-    auto rhs = [&](const float* val, const float* base, float a) {
+    auto rhs = [&](const float* val, const float* x, const float* mul, const float* base, float a, float* r) {
         split(N, [&](auto lpr) {
             constexpr int LPR = decltype(lpr)::value;
-            rhs_kernel<LPR><<<blocks_for(N * LPR), 256, 0, st>>>(p->SC, val, p->ca, base, a, p->ch_dinv, cf, p->cr, p->cd0);
+            rhs_kernel<LPR><<<blocks_for(N * LPR), 256, 0, st>>>(p->SC, val, x, mul, base, a, r);
         });
     };
-    rhs(p->vk, p->rp, spec.inv_pecn);
-    *nk += 2 + cheb_steps<float>(p->SC, p->va, p->ch_dinv, cf, CH_DEG, p->cr, p->cx, p->cd0, p->cd1, nullptr, p->ca, 1, 0, st);
-    rhs(p->vm, nullptr, spec.dt);
-    *nk += 2 + cheb_steps<float>(p->SC, p->va, p->ch_dinv, cf, CH_DEG, p->cr, p->cx, p->cd0, p->cd1, nullptr, p->ca, 1, 0, st);
+    auto solve = [&](const float* b, float* x) {   // (M + eps K)^{-1} b
+        return cheb<float>(p->SC, p->va, p->ch_dinv, cf, CH_DEG, b, p->cr, p->cx, p->cd0, p->cd1, nullptr, x, 1, 0, PrecondMean(), st);
+    };
+    rhs(p->vk, p->rm, p->iml, p->rp, spec.inv_pecn, p->cb);   // r_phi + K M_L^{-1} r_mu / (Pe Cn)
+    *nk += 1 + solve(p->cb, p->ca);
+    rhs(p->vm, p->ca, nullptr, nullptr, spec.dt, p->cb);      // dt M s
+    *nk += 2 + solve(p->cb, p->ca);
     split(N, [&](auto lpr) {
         constexpr int LPR = decltype(lpr)::value;
-        ch_store_kernel<LPR, TO><<<blocks_for(N * LPR), 256, 0, st>>>(p->SC, p->vk, NF, f, p->ca, p->rm, p->psi2, p->ml, spec.cn2, z);
+        ch_store_kernel<LPR, TO><<<blocks_for(N * LPR), 256, 0, st>>>(p->SC, p->vk, NF, f, p->ca, p->rm, p->psi2, p->iml, spec.cn2, z);
     });
     return cudaGetLastError();
 }
 template <class TO>
-cudaError_t enqueue(chns_mesh* m, const PrecondSpec& spec, const double* v, TO* z, cudaStream_t st, cudaStream_t side, int* nk) {
+cudaError_t enqueue(chns_mesh* m, const PrecondSpec& spec, TO* z, const PrecondMean& mean, cudaStream_t st, cudaStream_t side,
+                    int* nk) {
     PrecondWS* p = m->pre;
     const int D = m->dm.dim, NF = m->dm.nf;
     cudaError_t e = cudaSuccess;
@@ -965,9 +952,9 @@ cudaError_t enqueue(chns_mesh* m, const PrecondSpec& spec, const double* v, TO* 
         if (e == cudaSuccess) e = cudaStreamWaitEvent(side, p->fork, 0);
         if (e != cudaSuccess) return e;
     }
-    if (spec.ch) e = cahn_hilliard<TO>(m, spec, v, z, NF, D + 1, both ? side : st, nk);
+    if (spec.ch) e = cahn_hilliard<TO>(m, spec, z, NF, D + 1, both ? side : st, nk);
     if (e == cudaSuccess && spec.schur)
-        e = spec.mg ? vcycle<TO>(m, spec, v, z, NF, D, st, nk) : polynomial<TO>(m, spec, v, z, NF, D, st, nk);
+        e = spec.mg ? vcycle<TO>(m, spec, z, NF, D, mean, st, nk) : polynomial<TO>(m, spec, z, NF, D, mean, st, nk);
     if (both) {
         const cudaError_t e1 = cudaEventRecord(p->join, side);
         const cudaError_t e2 = cudaStreamWaitEvent(st, p->join, 0);
@@ -977,12 +964,12 @@ cudaError_t enqueue(chns_mesh* m, const PrecondSpec& spec, const double* v, TO* 
 }
 
 template <class TO>
-chns_status apply_any(chns_mesh* m, const PrecondSpec& spec, const double* v, TO* z, cudaStream_t s) {
+chns_status apply_any(chns_mesh* m, const PrecondSpec& spec, TO* z, const PrecondMean& mean, cudaStream_t s) {
     PrecondWS* p = m->pre;
     if (!p->no_graphs) {
         PrecondWS::Graph* hit = nullptr;
         for (auto& g : p->graph)
-            if (g.exec && g.v == (const void*)v && g.z == (const void*)z && g.to == sizeof(TO) && g.spec == spec) hit = &g;
+            if (g.exec && g.z == (const void*)z && g.to == sizeof(TO) && g.mean == (const void*)mean.out && g.spec == spec) hit = &g;
         if (!hit) {
             PrecondWS::Graph* slot = &p->graph[p->next];
             cudaGraph_t gr = nullptr;
@@ -990,7 +977,7 @@ chns_status apply_any(chns_mesh* m, const PrecondSpec& spec, const double* v, TO
             int nk = 0;
             bool ok = cudaStreamBeginCapture(p->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
             if (ok) {
-                ok = enqueue<TO>(m, spec, v, z, p->cap, p->cap2, &nk) == cudaSuccess;
+                ok = enqueue<TO>(m, spec, z, mean, p->cap, p->cap2, &nk) == cudaSuccess;
                 ok = (cudaStreamEndCapture(p->cap, &gr) == cudaSuccess) && ok && gr != nullptr;
                 if (ok) ok = cudaGraphInstantiate(&ex, gr, 0) == cudaSuccess;
                 if (gr) cudaGraphDestroy(gr);
@@ -1001,7 +988,7 @@ chns_status apply_any(chns_mesh* m, const PrecondSpec& spec, const double* v, TO
             } else {
                 if (slot->exec) cudaGraphExecDestroy(slot->exec);
                 slot->exec = ex;
-                slot->v = v;
+                slot->mean = mean.out;
                 slot->z = z;
                 slot->to = sizeof(TO);
                 slot->spec = spec;
@@ -1017,7 +1004,7 @@ chns_status apply_any(chns_mesh* m, const PrecondSpec& spec, const double* v, TO
         }
     }
     int nk = 0;
-    CHNS_CUDA(enqueue<TO>(m, spec, v, z, s, nullptr, &nk));
+    CHNS_CUDA(enqueue<TO>(m, spec, z, mean, s, nullptr, &nk));
     chns_count_launches(nk);
     return CHNS_OK;
 }
@@ -1063,8 +1050,8 @@ chns_status precond_prepare(chns_mesh* m, const PrecondSpec& spec, cudaStream_t 
         CHNS_CUDA(inc_build(L, s));
         CHNS_CUDA(sell_build<true>(L, p->SC, s));
         for (float** a : {&p->vm, &p->vk, &p->va}) CHNS_CUDA(alloc(a, p->SC.nnz));
-        for (float** a : {&p->ch_dinv, &p->ml, &p->rm, &p->rp, &p->ca, &p->cr, &p->cx, &p->cd0}) CHNS_CUDA(alloc(a, N));
-        ml_kernel<<<blocks_for(N), 256, 0, s>>>(N, m->d_nmass, p->ml);
+        for (float** a : {&p->ch_dinv, &p->iml, &p->rm, &p->rp, &p->cb, &p->ca, &p->cr, &p->cx, &p->cd0}) CHNS_CUDA(alloc(a, N));
+        iml_kernel<<<blocks_for(N), 256, 0, s>>>(N, m->d_nmass, p->iml);
         sell_values_kernel<true><<<blocks_for(p->SC.ns * 1024), 256, 0, s>>>(m->dm, p->SC, reference(m->dm.dim, false),
                                                                              reference(m->dm.dim, true), L.ip, L.inc, nullptr,
                                                                              p->vk, p->vm, nullptr, nullptr);
@@ -1125,11 +1112,18 @@ chns_status precond_setup(chns_mesh* m, const PrecondSpec& spec, const float* ce
 
 const unsigned int* precond_flags(const chns_mesh* m) { return m->pre->flags; }
 
-chns_status precond_apply(chns_mesh* m, const PrecondSpec& spec, const double* v, float* z, cudaStream_t s) {
-    return apply_any(m, spec, v, z, s);
+chns_status precond_apply(chns_mesh* m, const PrecondSpec& spec, float* z, const PrecondMean& mean, cudaStream_t s) {
+    return apply_any(m, spec, z, mean, s);
 }
-chns_status precond_apply(chns_mesh* m, const PrecondSpec& spec, const double* v, double* z, cudaStream_t s) {
-    return apply_any(m, spec, v, z, s);
+chns_status precond_apply(chns_mesh* m, const PrecondSpec& spec, double* z, const PrecondMean& mean, cudaStream_t s) {
+    return apply_any(m, spec, z, mean, s);
+}
+PrecondIn precond_inputs(const chns_mesh* m) {
+    PrecondIn in;
+    if (!m->pre->lv.empty()) in.p = m->pre->lv[0].b;
+    in.phi = m->pre->rp;
+    in.mu = m->pre->rm;
+    return in;
 }
 
 void precond_drop_graphs(chns_mesh* m) {
@@ -1146,7 +1140,7 @@ void precond_free(PrecondWS* p) {
         if (g.exec) cudaGraphExecDestroy(g.exec);
     for (auto& L : p->lv) level_free(L);
     sell_free(p->SC);
-    for (float* a : {p->vm, p->vk, p->va, p->ch_dinv, p->ml, p->rm, p->rp, p->ca, p->cr, p->cx, p->cd0, p->cd1}) cudaFree(a);
+    for (float* a : {p->vm, p->vk, p->va, p->ch_dinv, p->iml, p->rm, p->rp, p->cb, p->ca, p->cr, p->cx, p->cd0, p->cd1}) cudaFree(a);
     cudaFree(p->cf);
     cudaFree(p->kmax);
     cudaFree(p->flags);

@@ -29,10 +29,23 @@ chns_status precond_prepare(chns_mesh* m, const PrecondSpec& spec, cudaStream_t 
 chns_status precond_setup(chns_mesh* m, const PrecondSpec& spec, const float* ce, const float* psi2, cudaStream_t s);
 // device word, zeroed by precond_setup: bit 0 Schur bound, bit 1 Cahn-Hilliard bound not finite
 const unsigned int* precond_flags(const chns_mesh* m);
-// Overwrites the pressure (schur) and phi, mu (ch) rows of z with the preconditioned rows of the
-// FP64 vector v.  Replayed from a CUDA graph per (v, z, spec).
-chns_status precond_apply(chns_mesh* m, const PrecondSpec& spec, const double* v, float* z, cudaStream_t s);
-chns_status precond_apply(chns_mesh* m, const PrecondSpec& spec, const double* v, double* z, cudaStream_t s);
+// Compact inputs (FP32, one value per node) that the caller writes before every application: the
+// pressure, phi and mu rows of the vector.  Overwritten by the application.
+struct PrecondIn {
+    float *p = nullptr, *phi = nullptr, *mu = nullptr;
+};
+PrecondIn precond_inputs(const chns_mesh* m);
+// m_p^T z_p: formed with the pressure result (null out: not wanted)
+struct PrecondMean {
+    const double* nmass = nullptr;
+    double* partials = nullptr;        // N / 64 + 64
+    unsigned int* counter = nullptr;   // zero
+    double* out = nullptr;
+};
+// Writes the pressure (schur) and phi, mu (ch) rows of z from the inputs.  Replayed from a CUDA
+// graph per (z, mean, spec).
+chns_status precond_apply(chns_mesh* m, const PrecondSpec& spec, float* z, const PrecondMean& mean, cudaStream_t s);
+chns_status precond_apply(chns_mesh* m, const PrecondSpec& spec, double* z, const PrecondMean& mean, cudaStream_t s);
 // Captured graphs hold the callers' vectors: drop them when those are freed.
 void precond_drop_graphs(chns_mesh* m);
 void precond_free(PrecondWS* p);

@@ -22,13 +22,14 @@
 
 #include "block_jacobi.h"
 #include "chns_internal.h"
+#include "krylov.h"
 #include "precond.h"
 #include "reduce.cuh"
 
 struct SolverWS {
     int restart = 0;
-    int64_t n = 0, N = 0;
-    double* V = nullptr;     // (restart + 1) * n Arnoldi basis
+    int64_t n = 0, N = 0, ld = 0;
+    double* V = nullptr;     // (restart + 1) * ld Arnoldi basis (ld: n rounded up to 16 bytes)
     double* w = nullptr;     // n
     double* R = nullptr;     // n residual
     double* dU = nullptr;    // n Newton update
@@ -51,20 +52,14 @@ struct SolverWS {
     cudaEvent_t ev[16] = {};  // J x, preconditioner build / apply and Gram-Schmidt timing (two sets
                               // of J x / apply events alternate between Arnoldi steps)
     float* ce = nullptr;     // E element coefficients of the pressure Schur approximation
-    cudaStream_t cap = nullptr;   // capture stream of the Gram-Schmidt graphs
-    bool no_graphs = false;
-    // CUDA graphs of the Gram-Schmidt sequence of Arnoldi step j (its kernels take k = j + 1
-    // and fixed workspace pointers), captured at first use
-    cudaGraphExec_t orth_exec[257] = {};
-    double* part = nullptr;  // per-block partials of the fused orthogonalisation reductions
+    double* part = nullptr;  // per-block partials of the Gram-Schmidt reductions
+    double* mpart = nullptr; // and of the pressure mean
+    unsigned int* counter = nullptr;   // blocks that finished: Gram-Schmidt, pressure mean
     float* ch_psi2 = nullptr;  // psi''(phi~) at the nodes (Cahn-Hilliard block)
 };
 
 void chns_solver_ws_free(SolverWS* ws) {
     if (!ws) return;
-    for (auto& g : ws->orth_exec)
-        if (g) cudaGraphExecDestroy(g);
-    if (ws->cap) cudaStreamDestroy(ws->cap);
     cudaFree(ws->V);
     cudaFree(ws->w);
     cudaFree(ws->R);
@@ -86,6 +81,8 @@ void chns_solver_ws_free(SolverWS* ws) {
     cudaFree(ws->sc);
     cudaFree(ws->ce);
     cudaFree(ws->part);
+    cudaFree(ws->mpart);
+    cudaFree(ws->counter);
     cudaFree(ws->ch_psi2);
     if (ws->hsc) cudaFreeHost(ws->hsc);
     for (auto& e : ws->ev)
@@ -96,7 +93,6 @@ void chns_solver_ws_free(SolverWS* ws) {
 namespace {
 
 constexpr int MAXSC = 1024;
-constexpr int ORTH_MAX_BX = 1024;   // row blocks of the fused orthogonalisation kernels
 
 chns_status ensure_ws(chns_mesh* m, int restart) {
     SolverWS* ws = m->ws;
@@ -110,12 +106,13 @@ chns_status ensure_ws(chns_mesh* m, int restart) {
     ws->restart = restart;
     ws->N = m->dm.N;
     ws->n = m->dm.N * m->dm.nf;
+    ws->ld = (ws->n + 1) / 2 * 2;
     const size_t n = (size_t)ws->n, nb = (size_t)m->dm.N * m->dm.nf * m->dm.nf;
     cudaError_t e = cudaSuccess;
     auto A = [&](void** p, size_t bytes) {
         if (e == cudaSuccess) e = cudaMalloc(p, bytes);
     };
-    A((void**)&ws->V, (size_t)(restart + 1) * n * sizeof(double));
+    A((void**)&ws->V, (size_t)(restart + 1) * ws->ld * sizeof(double));
     A((void**)&ws->w, n * sizeof(double));
     A((void**)&ws->R, n * sizeof(double));
     A((void**)&ws->dU, n * sizeof(double));
@@ -135,7 +132,10 @@ chns_status ensure_ws(chns_mesh* m, int restart) {
     A((void**)&ws->Pinv64, nb * sizeof(double));
     A((void**)&ws->sc, MAXSC * sizeof(double));
     A((void**)&ws->ce, (size_t)m->dm.E * sizeof(float));
-    A((void**)&ws->part, (size_t)ORTH_MAX_BX * (MAXSC / 32 + 1) * 9 * sizeof(double));
+    A((void**)&ws->part, (size_t)33 * 16 * chns_num_sms() * sizeof(double));   // 33 numbers of up to 16 blocks per SM
+    A((void**)&ws->mpart, (size_t)(m->dm.N / 64 + 64) * sizeof(double));
+    A((void**)&ws->counter, 2 * sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMemset(ws->counter, 0, 2 * sizeof(unsigned int));
     A((void**)&ws->ch_psi2, (size_t)m->dm.N * sizeof(float));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&ws->hsc, MAXSC * sizeof(double));
     for (auto& ev : ws->ev)
@@ -161,149 +161,6 @@ __global__ void to64_kernel(const float* __restrict__ a, double* __restrict__ b,
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         b[i] = (double)a[i];
 }
-// w -= sum_{j<k} h[j] V_j  (h in device memory)
-__global__ void gs_update_kernel(const double* __restrict__ V, int64_t ld, int k, const double* __restrict__ h,
-                                 double* __restrict__ w, int64_t n) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        double s = w[i];
-        for (int j = 0; j < k; ++j) s -= h[j] * V[(size_t)j * ld + i];
-        w[i] = s;
-    }
-}
-// Fused h = V^T w for all k basis vectors (blockIdx.y picks 8 of them) and, in chunk 0,
-// also w . w: partials[(chunk * gridDim.x + block) * 9 + j].  The 8 dot products of a
-// warp are reduced by recursive halving (each exchange level hands half of the
-// remaining values to the partner lane): 9 FP64 shuffle-adds per warp instead of 40,
-// which matters because every FP64 add runs on the narrow FP64 pipe.
-__global__ void orth_dots_kernel(const double* __restrict__ V, int64_t ld, int k, const double* __restrict__ w,
-                                 int64_t n, double* __restrict__ partials, const double* __restrict__ pred) {
-    if (pred && pred[0] == 0.0) return;   // second pass not needed (decided on the device)
-    const int chunk = blockIdx.y;
-    const int j0 = chunk * 8;
-    const int kk = min(8, k - j0);
-    double acc[8];
-    double nrm = 0.0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[j] = 0.0;
-    const double* Vc = V + (size_t)j0 * ld;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double wi = w[i];
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            if (j < kk) acc[j] += Vc[(size_t)j * ld + i] * wi;
-        if (chunk == 0) nrm += wi * wi;
-    }
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // 8 -> 4 values (lane bit 4 keeps the upper half), 4 -> 2 (bit 3), 2 -> 1 (bit 2)
-    double t4[4], t2[2];
-    {
-        const bool up = lane & 16;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const double keep = up ? acc[4 + t] : acc[t];
-            const double give = up ? acc[t] : acc[4 + t];
-            t4[t] = keep + __shfl_xor_sync(full, give, 16);
-        }
-    }
-    {
-        const bool up = lane & 8;
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            const double keep = up ? t4[2 + t] : t4[t];
-            const double give = up ? t4[t] : t4[2 + t];
-            t2[t] = keep + __shfl_xor_sync(full, give, 8);
-        }
-    }
-    const bool up4 = lane & 4;
-    double t1 = (up4 ? t2[1] : t2[0]) + __shfl_xor_sync(full, up4 ? t2[0] : t2[1], 4);
-    t1 += __shfl_xor_sync(full, t1, 2);
-    t1 += __shfl_xor_sync(full, t1, 1);
-    // lane holds the warp sum of value ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)
-    __shared__ double sred[32][9];
-    if ((lane & 3) == 0) sred[warp][((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] = t1;
-    if (chunk == 0) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) nrm += __shfl_xor_sync(full, nrm, off);
-        if (lane == 0) sred[warp][8] = nrm;
-    }
-    __syncthreads();
-    if (threadIdx.x < 9) {
-        double v = 0.0;
-        if (threadIdx.x < 8 || chunk == 0)
-            for (int w2 = 0; w2 < (int)(blockDim.x >> 5); ++w2) v += sred[w2][threadIdx.x];
-        partials[((size_t)chunk * gridDim.x + blockIdx.x) * 9 + threadIdx.x] = v;
-    }
-}
-// out[j] = sum over row blocks (one block per chunk, one warp per value), out_norm = w.w
-__global__ void orth_dots_final_kernel(const double* __restrict__ partials, int nbx, int k, double* __restrict__ out,
-                                       double* __restrict__ out_norm, const double* __restrict__ pred) {
-    if (pred && pred[0] == 0.0) return;
-    const int chunk = blockIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;   // 9 warps
-    const int j = warp;
-    if (j >= 9) return;
-    if (j < 8 && chunk * 8 + j >= k) return;
-    if (j == 8 && chunk != 0) return;
-    double v = 0.0;
-    for (int b = lane; b < nbx; b += 32) v += partials[((size_t)chunk * nbx + b) * 9 + j];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (lane == 0) {
-        if (j < 8) out[chunk * 8 + j] = v;
-        else out_norm[0] = v;
-    }
-}
-// w -= sum_{j<k} h[j] V_j, and per-block partials of the new w . w
-__global__ void gs_update_norm_kernel(const double* __restrict__ V, int64_t ld, int k, const double* __restrict__ h,
-                                      double* __restrict__ w, int64_t n, double* __restrict__ partials,
-                                      const double* __restrict__ pred) {
-    if (pred && pred[0] == 0.0) return;
-    double acc[1] = {0.0};
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        double s = w[i];
-        for (int j = 0; j < k; ++j) s -= h[j] * V[(size_t)j * ld + i];
-        w[i] = s;
-        acc[0] += s * s;
-    }
-    block_reduce_store<1>(acc, partials);
-}
-// Second Gram-Schmidt pass only on severe cancellation (|w'|^2 < 0.01 |w|^2 after the
-// first pass; on GB300 every pass is bound by the FP64 pipe): the flag goes to sc[605]
-// for the predicated second-pass kernels; when the pass is skipped its coefficients
-// sc[256..256+k) are zeroed and the norm sc[601] is carried to sc[603], so the host
-// always reads h = h1 + h2 and the final |w|^2 from the same slots.
-__global__ void reorth_decide_kernel(double* __restrict__ sc, int k) {
-    const bool again = sc[601] < 0.01 * sc[600];
-    if (!again)
-        for (int i = threadIdx.x; i < k; i += blockDim.x) sc[256 + i] = 0.0;
-    if (threadIdx.x == 0) {
-        sc[605] = again ? 1.0 : 0.0;
-        if (!again) sc[603] = sc[601];
-    }
-}
-// final_reduce_kernel for one component (same fixed order), skipped when pred[0] == 0
-__global__ void final_reduce1_pred_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ out,
-                                          const double* __restrict__ pred) {
-    if (pred && pred[0] == 0.0) return;
-    __shared__ double sh[256];
-    double v = 0.0;
-    for (int i = threadIdx.x; i < nblocks; i += blockDim.x) v += partials[i];
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int st = 128; st > 0; st >>= 1) {
-        if ((int)threadIdx.x < st) sh[threadIdx.x] += sh[threadIdx.x + st];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[0] = sh[0];
-}
-// next Arnoldi vector v = w / sqrt(nrm[0]) (zero on breakdown, which the host reports)
-__global__ void scale_next_kernel(const double* __restrict__ w, double* __restrict__ v, int64_t n,
-                                  const double* __restrict__ nrm) {
-    const double a = nrm[0] > 0.0 ? 1.0 / sqrt(nrm[0]) : 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        v[i] = a * w[i];
-}
 // sum_n m_n (a + b - c)[n*NF + f] into per-block partials (the phi-mass change of a
 // Newton update: a = U, b = dU, c = U^k)
 __global__ void field_mass3_kernel(const double* __restrict__ m, const double* __restrict__ a,
@@ -316,27 +173,11 @@ __global__ void field_mass3_kernel(const double* __restrict__ m, const double* _
     }
     block_reduce_store<1>(acc, partials);
 }
-// u = sum_{j<k} y[j] V_j (y host-provided via device scalars)
-__global__ void combine_kernel(const double* __restrict__ V, int64_t ld, int k, const double* __restrict__ y,
-                               double* __restrict__ u, int64_t n) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int j = 0; j < k; ++j) s += y[j] * V[(size_t)j * ld + i];
-        u[i] = s;
-    }
-}
-// y = s .* x (FP32 or FP64 x)
+// y = a s .* x
 template <class T>
-__global__ void scale_vec_kernel(const T* x, const double* __restrict__ sv, double* y,
-                                 int64_t n) {
+__global__ void scale_vec_kernel(const T* x, const double* __restrict__ sv, double* y, double a, int64_t n) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        y[i] = sv[i] * (double)x[i];
-}
-// y = x .* d (d = 1/S, stored, so no FP64 division)
-__global__ void unscale_kernel(const double* __restrict__ x, const double* __restrict__ d, double* __restrict__ y,
-                               int64_t n) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        y[i] = x[i] * d[i];
+        y[i] = a * (sv[i] * (double)x[i]);
 }
 __global__ void axpy_kernel(double a, const double* __restrict__ x, double* __restrict__ y, int64_t n) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -446,22 +287,67 @@ __global__ void pc_invert_kernel(DevMesh m, const TB* __restrict__ blk, TI* __re
         for (int j = 0; j < NF; ++j) inv[((size_t)n * NF + i) * NF + j] = (TI)A[i][NF + j];
 }
 
-// z = P^{-1} v per node (FP64 input; output type TO, arithmetic in the storage type's
-// precision promoted to FP64 for the final update)
-template <class TI, class TO>
-__global__ void pc_apply_kernel(int64_t N, int NF, const TI* __restrict__ inv, const double* __restrict__ v,
-                                TO* __restrict__ z) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    // arithmetic in the precision the blocks are stored in (FP32 for the mixed path)
-    TI x[6];
-    for (int j = 0; j < NF; ++j) x[j] = (TI)v[(size_t)n * NF + j];
-    for (int i = 0; i < NF; ++i) {
-        TI s = TI(0);
-        for (int j = 0; j < NF; ++j) s += inv[((size_t)n * NF + i) * NF + j] * x[j];
-        z[(size_t)n * NF + i] = (TO)s;
+// First part of a preconditioner application: x = scale * v .* Sd (either may be null), z = P^{-1} x
+// with the nodal blocks (P^{-T}: TRANS) in the precision they are stored in, and the rows that are
+// preconditioned as scalar operators (mask 1: p; 2: phi, mu) to their compact FP32 inputs instead.
+// One thread per row: the n_f entries of a row of blocks are read by its thread, neighbouring rows
+// by neighbouring threads.  (64^3, FP32: 15 us; one thread per node, behind a pass that scaled v:
+// 6.8 + 25.6 us.)
+constexpr int PC_NODES = 32;
+template <int NF, bool TRANS, class TI, class TO>
+__global__ void __launch_bounds__(PC_NODES * NF) pc_first_kernel(int64_t N, int mask, const TI* __restrict__ inv,
+                                                                 const double* __restrict__ v,
+                                                                 const double* __restrict__ scale,
+                                                                 const double* __restrict__ Sd, TO* __restrict__ z,
+                                                                 PrecondIn in) {
+    constexpr int D = NF - 3;
+    __shared__ TI xs[PC_NODES * NF];
+    __shared__ TI bl[TRANS ? PC_NODES * NF * NF : 1];
+    const int64_t node0 = (int64_t)blockIdx.x * PC_NODES;
+    const int ln = threadIdx.x / NF, row = threadIdx.x % NF;
+    const int64_t node = node0 + ln, i = node0 * NF + threadIdx.x;
+    const bool ok = node < N;
+    double x = 0.0;
+    if (ok) {
+        x = v[i];
+        if (scale) x *= scale[0];
+        if (Sd) x *= Sd[i];
     }
+    xs[threadIdx.x] = (TI)x;
+    if (TRANS) {
+        const int64_t end = N * NF * NF;
+        for (int t = threadIdx.x; t < PC_NODES * NF * NF; t += PC_NODES * NF)
+            bl[t] = node0 * NF * NF + t < end ? inv[node0 * NF * NF + t] : TI(0);
+    }
+    __syncthreads();
+    if (!ok) return;
+    if (row == D && (mask & 1)) {
+        in.p[node] = (float)x;
+        return;
+    }
+    if (row > D && (mask & 2)) {
+        (row == D + 1 ? in.phi : in.mu)[node] = (float)x;
+        return;
+    }
+    TI s = TI(0);
+#pragma unroll
+    for (int j = 0; j < NF; ++j) {
+        const TI a = TRANS ? bl[(ln * NF + j) * NF + row] : inv[(size_t)i * NF + j];
+        s += a * xs[ln * NF + j];
+    }
+    z[i] = (TO)s;
 }
+template <bool TRANS, class TI, class TO>
+void launch_pc_first(const chns_mesh* m, int mask, const TI* inv, const double* v, const double* scale, const double* Sd, TO* z,
+                     cudaStream_t s) {
+    const int64_t N = m->dm.N;
+    const unsigned g = (unsigned)((N + PC_NODES - 1) / PC_NODES);
+    const PrecondIn in = mask ? precond_inputs(m) : PrecondIn();
+    if (m->dm.nf == 5) pc_first_kernel<5, TRANS, TI, TO><<<g, PC_NODES * 5, 0, s>>>(N, mask, inv, v, scale, Sd, z, in);
+    else pc_first_kernel<6, TRANS, TI, TO><<<g, PC_NODES * 6, 0, s>>>(N, mask, inv, v, scale, Sd, z, in);
+    chns_count_launches(1);
+}
+__global__ void set_scalar_kernel(double* p, double v) { *p = v; }
 
 // ---------------- initial chemical potential (mass-matrix CG) ----------------
 // b_a = sum_q |J| (N_a psi'(phi_q) + Cn^2 grad N_a . grad phi_q)  and  y = M x, with the
@@ -668,26 +554,22 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
     std::vector<double> H((size_t)(mres + 1) * mres), cs(mres), sn(mres), gv(mres + 1), y(mres);
     double r0 = 0.0, rn = 0.0;
     chns_status result = CHNS_OK;
-    // one classical Gram-Schmidt pass against V_0..V_{k-1}: h -> hdev[0..k), |w|^2 before
-    // -> nrm_before, |w|^2 after -> nrm_after (all device scalars); with pred, every kernel
-    // of the pass returns at once when pred[0] == 0
-    auto orth_pass = [&](cudaStream_t st, int k, double* hdev, double* nrm_before, double* nrm_after,
-                         const double* pred) {
-        int nbx = c.g < ORTH_MAX_BX ? c.g : ORTH_MAX_BX;
-        const int nch = (k + 7) / 8;
-        orth_dots_kernel<<<dim3(nbx, nch), 256, 0, st>>>(ws->V, c.n, k, ws->w, c.n, ws->part, pred);
-        orth_dots_final_kernel<<<nch, 288, 0, st>>>(ws->part, nbx, k, hdev, nrm_before, pred);
-        gs_update_norm_kernel<<<nbx, 256, 0, st>>>(ws->V, c.n, k, hdev, ws->w, c.n, m->d_partials, pred);
-        final_reduce1_pred_kernel<<<1, 256, 0, st>>>(m->d_partials, nbx, nrm_after, pred);
-    };
-    // Gram-Schmidt of Arnoldi step j with device-decided re-orthogonalisation, the next
-    // Arnoldi vector and the read-back of the Hessenberg column: 10 kernels and a copy
-    auto orth_enqueue = [&](cudaStream_t st, int j) {
-        orth_pass(st, j + 1, ws->sc, ws->sc + 600, ws->sc + 601, nullptr);
-        reorth_decide_kernel<<<1, 256, 0, st>>>(ws->sc, j + 1);
-        orth_pass(st, j + 1, ws->sc + 256, ws->sc + 602, ws->sc + 603, ws->sc + 605);
-        scale_next_kernel<<<c.g, 256, 0, st>>>(ws->w, ws->V + (size_t)(j + 1) * c.n, c.n, ws->sc + 603);
-        cudaMemcpyAsync(ws->hsc, ws->sc, 606 * sizeof(double), cudaMemcpyDeviceToHost, st);
+    // m_p^T z of the pin-mode-2 operator J + u m_p^T / |Omega|: formed with the pressure rows of z by
+    // the pressure preconditioner, or by a pass of its own
+    PrecondMean pmn;
+    if (pin == 2) {
+        pmn.nmass = m->d_nmass;
+        pmn.partials = ws->mpart;
+        pmn.counter = ws->counter + 1;
+        pmn.out = ws->sc + SC_MEAN;
+    }
+    // Gram-Schmidt of Arnoldi step j on w = S J z (+ the rank-one term), with device-decided
+    // re-orthogonalisation, and the read-back of the Hessenberg column
+    const double thr = 0.01;
+    auto orth_enqueue = [&](cudaStream_t st, int j) -> int {
+        const double* mean = pin == 2 ? ws->sc + SC_MEAN : nullptr;
+        const krylov::Source src{mixed ? ws->y32 : nullptr, mixed ? nullptr : ws->t64, ws->S, mean, 1.0 / m->volume, NF, D};
+        return krylov::orthogonalise(ws->V, ws->ld, j + 1, src, c.n, ws->sc, thr, ws->hsc, ws->part, ws->counter, st);
     };
     auto build_pc = [&]() -> chns_status {
         CHNS_CUDA(cudaEventRecord(ws->ev[2], c.s));
@@ -713,12 +595,12 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
         CHNS_CUDA(cudaEventRecord(ws->ev[3], c.s));
         return CHNS_OK;
     };
-    // m_p^T v / |Omega| term of the pin-mode-2 operator: sum_n m_n v_p[n] into sc[610]
+    // m_p^T v of vectors that do not come from the pressure preconditioner
     const double inv_vol = 1.0 / m->volume;
     const int nbm = c.g < 1024 ? c.g : 1024;
     auto pmean = [&](const auto* v) {
         { field_mass_kernel<<<nbm, 256, 0, c.s>>>(m->d_nmass, v, NF, D, m->dm.N, m->d_partials); chns_count_launches(1); }
-        { final_reduce_kernel<<<1, 256, 0, c.s>>>(m->d_partials, nbm, 1, ws->sc + 610); chns_count_launches(1); }
+        { final_reduce_kernel<<<1, 256, 0, c.s>>>(m->d_partials, nbm, 1, ws->sc + SC_MEAN); chns_count_launches(1); }
     };
     bool pc_pending = false;
     double eta_prev = 0.0, rn_prev = 0.0;   // previous forcing term and residual (Eisenstat-Walker)
@@ -732,7 +614,7 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
             pc_pending = true;
             { copy64_kernel<<<c.g, 256, 0, c.s>>>(ws->S, ws->S0, c.n); chns_count_launches(1); }
         }
-        { scale_vec_kernel<double><<<c.g, 256, 0, c.s>>>(ws->R, ws->S0, ws->SR, c.n); chns_count_launches(1); }
+        { scale_vec_kernel<double><<<c.g, 256, 0, c.s>>>(ws->R, ws->S0, ws->SR, 1.0, c.n); chns_count_launches(1); }
         if ((st = dot_host(c, ws->SR, ws->SR, &rn)) != CHNS_OK) return st;
         if (schur && (st = pc_flags_check(c)) != CHNS_OK) return st;
         unsigned int flag = 0;
@@ -758,12 +640,11 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
         CHNS_CUDA(cudaMemsetAsync(ws->dU, 0, c.n * sizeof(double), c.s));
         double rnorm = rn;
         int kry = 0;
-        // r = -S R (S: row equilibration of this linearisation)
-        { scale_vec_kernel<double><<<c.g, 256, 0, c.s>>>(ws->R, ws->S, ws->w, c.n); chns_count_launches(1); }
-        { axpby_kernel<<<c.g, 256, 0, c.s>>>(0.0, ws->w, -1.0, ws->w, c.n); chns_count_launches(1); }
+        // r = -S R (S: row equilibration of this linearisation), in slot 0 of the basis
+        { scale_vec_kernel<double><<<c.g, 256, 0, c.s>>>(ws->R, ws->S, ws->V, -1.0, c.n); chns_count_launches(1); }
         {
             double bb;
-            if ((st = dot_host(c, ws->w, ws->w, &bb)) != CHNS_OK) return st;
+            if ((st = dot_host(c, ws->V, ws->V, &bb)) != CHNS_OK) return st;
             if (schur && (st = pc_flags_check(c)) != CHNS_OK) return st;
             rnorm = std::sqrt(bb);
         }
@@ -788,47 +669,38 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
         const double eta = std::max(eta_k, std::min(0.5, 0.1 * target / rn));
         eta_prev = eta_k;
         rn_prev = rn;
-        // w = S J M^{-1} S^{-1} V_j (similarity scaling: the eigenvalues are those of J M^{-1});
-        // the J x / apply timing events come from set es (two sets alternate, so the next
-        // vector's application can be queued before this one's events are read)
+        // z = M^{-1} S^{-1} v_j and y = J z; w = S y (similarity scaling: the eigenvalues of S J M^{-1}
+        // S^{-1} are those of J M^{-1}) is formed by the dot pass that reads it.  The J x / apply
+        // timing events come from set es (two sets alternate, so the next vector's application can
+        // be queued before this one's events are read)
         auto apply_op = [&](int j, int es) -> chns_status {
-            const double* Vj = ws->V + (size_t)j * c.n;
+            const double *Vj = ws->V + (size_t)j * ws->ld, *sj = ws->sc + SC_SCALE + j;
             cudaEvent_t* E = ws->ev + 8 * es;
             CHNS_CUDA(cudaEventRecord(E[4], c.s));
-            { unscale_kernel<<<c.g, 256, 0, c.s>>>(Vj, ws->Sd, ws->SR, c.n); chns_count_launches(1); }
             if (mixed) {
-                { pc_apply_kernel<float, float><<<gN, 128, 0, c.s>>>(m->dm.N, NF, ws->Pinv32, ws->SR, ws->z32); chns_count_launches(1); }
-                if (schur && (st = precond_apply(m, spec, ws->SR, ws->z32, c.s)) != CHNS_OK) return st;
-                if (pin == 2) pmean(ws->z32);
+                launch_pc_first<false>(m, pcmask, ws->Pinv32, Vj, sj, ws->Sd, ws->z32, c.s);
+                if (schur && (st = precond_apply(m, spec, ws->z32, pmn, c.s)) != CHNS_OK) return st;
+                if (pin == 2 && !schur) pmean(ws->z32);
                 CHNS_CUDA(cudaEventRecord(E[5], c.s));
                 CHNS_CUDA(cudaEventRecord(E[0], c.s));
                 CHNS_CUDA(launch_jvp32(m, pc, ws->Uo32, ws->Us32, ws->z32, ws->y32, pin, c.s));
-                CHNS_CUDA(cudaEventRecord(E[1], c.s));
-                if (pin == 2)
-                    { scale_vec_pmean_kernel<float><<<c.g, 256, 0, c.s>>>(ws->y32, ws->S, ws->w, c.n, NF, D, ws->sc + 610, inv_vol); chns_count_launches(1); }
-                else
-                    { scale_vec_kernel<float><<<c.g, 256, 0, c.s>>>(ws->y32, ws->S, ws->w, c.n); chns_count_launches(1); }
             } else {
-                { pc_apply_kernel<double, double><<<gN, 128, 0, c.s>>>(m->dm.N, NF, ws->Pinv64, ws->SR, ws->z64); chns_count_launches(1); }
-                if (schur && (st = precond_apply(m, spec, ws->SR, ws->z64, c.s)) != CHNS_OK) return st;
-                if (pin == 2) pmean(ws->z64);
+                launch_pc_first<false>(m, pcmask, ws->Pinv64, Vj, sj, ws->Sd, ws->z64, c.s);
+                if (schur && (st = precond_apply(m, spec, ws->z64, pmn, c.s)) != CHNS_OK) return st;
+                if (pin == 2 && !schur) pmean(ws->z64);
                 CHNS_CUDA(cudaEventRecord(E[5], c.s));
                 CHNS_CUDA(cudaEventRecord(E[0], c.s));
                 CHNS_CUDA(launch_jvp64(m, pc, U_old, U, ws->z64, ws->t64, pin, c.s));
-                CHNS_CUDA(cudaEventRecord(E[1], c.s));
-                if (pin == 2)
-                    { scale_vec_pmean_kernel<double><<<c.g, 256, 0, c.s>>>(ws->t64, ws->S, ws->w, c.n, NF, D, ws->sc + 610, inv_vol); chns_count_launches(1); }
-                else
-                    { scale_vec_kernel<double><<<c.g, 256, 0, c.s>>>(ws->t64, ws->S, ws->w, c.n); chns_count_launches(1); }
             }
+            CHNS_CUDA(cudaEventRecord(E[1], c.s));
             CHNS_CUDA(cudaGetLastError());
             S.jvp_calls++;
             return CHNS_OK;
         };
         while (true) {
-            // V0 = r / ||r||
+            // v_0 = r / ||r||: r is in slot 0
             double beta = rnorm;
-            { axpby_kernel<<<c.g, 256, 0, c.s>>>(1.0 / beta, ws->w, 0.0, ws->V, c.n); chns_count_launches(1); }
+            { set_scalar_kernel<<<1, 1, 0, c.s>>>(ws->sc + SC_SCALE, 1.0 / beta); chns_count_launches(1); }
             std::fill(gv.begin(), gv.end(), 0.0);
             gv[0] = beta;
             int j = 0;
@@ -839,33 +711,8 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
                 // classical Gram-Schmidt with selective re-orthogonalisation (decided on the
                 // device) and the next Arnoldi vector, all queued without a host round trip
                 CHNS_CUDA(cudaEventRecord(ws->ev[6], c.s));
-                {
-                    // replayed from a CUDA graph of this j once captured (the launches are short)
-                    bool done_g = false;
-                    if (!ws->no_graphs && j < 257) {
-                        if (!ws->orth_exec[j]) {
-                            cudaGraph_t gr = nullptr;
-                            cudaGraphExec_t ex = nullptr;
-                            bool ok = ws->cap || cudaStreamCreateWithFlags(&ws->cap, cudaStreamNonBlocking) == cudaSuccess;
-                            if (ok) ok = cudaStreamBeginCapture(ws->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-                            if (ok) {
-                                orth_enqueue(ws->cap, j);
-                                ok = cudaStreamEndCapture(ws->cap, &gr) == cudaSuccess && gr != nullptr;
-                                if (ok) ok = cudaGraphInstantiate(&ex, gr, 0) == cudaSuccess;
-                                if (gr) cudaGraphDestroy(gr);
-                            }
-                            if (ok) ws->orth_exec[j] = ex;
-                            else { (void)cudaGetLastError(); ws->no_graphs = true; }
-                        }
-                        if (ws->orth_exec[j]) {
-                            CHNS_CUDA(cudaGraphLaunch(ws->orth_exec[j], c.s));
-                            done_g = true;
-                        }
-                    }
-                    if (!done_g) orth_enqueue(c.s, j);
-                    chns_count_launches(10);
-                    CHNS_CUDA(cudaGetLastError());
-                }
+                chns_count_launches(orth_enqueue(c.s, j));
+                CHNS_CUDA(cudaGetLastError());
                 CHNS_CUDA(cudaEventRecord(ws->ev[7], c.s));
                 CHNS_CUDA(cudaEventRecord(ws->ev[10], c.s));
                 // queue the next vector's operator application before reading the scalars, so
@@ -889,8 +736,8 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
                         pc_pending = false;
                     }
                 }
-                const double hn = std::sqrt(ws->hsc[603]);
-                for (int i = 0; i <= j; ++i) H[(size_t)i * mres + j] = ws->hsc[i] + ws->hsc[256 + i];
+                const double hn = std::sqrt(ws->hsc[SC_NA]);
+                for (int i = 0; i <= j; ++i) H[(size_t)i * mres + j] = ws->hsc[i];
                 H[(size_t)(j + 1) * mres + j] = hn;
                 if (!std::isfinite(hn)) { chns_set_error("non-finite Arnoldi vector"); S.reason = CHNS_EBREAKDOWN; result = CHNS_EBREAKDOWN; break; }
                 // Givens rotations
@@ -925,13 +772,11 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
             }
             std::memcpy(ws->hsc, y.data(), k * sizeof(double));
             CHNS_CUDA(cudaMemcpyAsync(ws->sc, ws->hsc, k * sizeof(double), cudaMemcpyHostToDevice, c.s));
-            { combine_kernel<<<c.g, 256, 0, c.s>>>(ws->V, c.n, k, ws->sc, ws->t64, c.n); chns_count_launches(1); }
-            { unscale_kernel<<<c.g, 256, 0, c.s>>>(ws->t64, ws->Sd, ws->SR, c.n); chns_count_launches(1); }
-            if (mixed)
-                { pc_apply_kernel<float, double><<<gN, 128, 0, c.s>>>(m->dm.N, NF, ws->Pinv32, ws->SR, ws->z64); chns_count_launches(1); }
-            else
-                { pc_apply_kernel<double, double><<<gN, 128, 0, c.s>>>(m->dm.N, NF, ws->Pinv64, ws->SR, ws->z64); chns_count_launches(1); }
-            if (schur && (st = precond_apply(m, spec, ws->SR, ws->z64, c.s)) != CHNS_OK) return st;
+            krylov::combine(ws->V, ws->ld, k, ws->sc, ws->sc + SC_SCALE, ws->SR, c.n, c.s);
+            chns_count_launches(1);
+            if (mixed) launch_pc_first<false>(m, pcmask, ws->Pinv32, ws->SR, nullptr, ws->Sd, ws->z64, c.s);
+            else launch_pc_first<false>(m, pcmask, ws->Pinv64, ws->SR, nullptr, ws->Sd, ws->z64, c.s);
+            if (schur && (st = precond_apply(m, spec, ws->z64, PrecondMean(), c.s)) != CHNS_OK) return st;
             { axpy_kernel<<<c.g, 256, 0, c.s>>>(1.0, ws->z64, ws->dU, c.n); chns_count_launches(1); }
             CHNS_CUDA(cudaGetLastError());
             if (done || kry >= o->max_krylov) break;
@@ -951,12 +796,12 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
             { axpby_kernel<<<c.g, 256, 0, c.s>>>(-1.0, ws->R, -1.0, ws->w, c.n); chns_count_launches(1); }
             if (pin == 2) {
                 pmean(ws->dU);
-                { scale_vec_pmean_kernel<double><<<c.g, 256, 0, c.s>>>(ws->w, ws->S, ws->w, c.n, NF, D, ws->sc + 610, -inv_vol); chns_count_launches(1); }
+                { scale_vec_pmean_kernel<double><<<c.g, 256, 0, c.s>>>(ws->w, ws->S, ws->V, c.n, NF, D, ws->sc + SC_MEAN, -inv_vol); chns_count_launches(1); }
             } else {
-                { scale_vec_kernel<double><<<c.g, 256, 0, c.s>>>(ws->w, ws->S, ws->w, c.n); chns_count_launches(1); }
+                { scale_vec_kernel<double><<<c.g, 256, 0, c.s>>>(ws->w, ws->S, ws->V, 1.0, c.n); chns_count_launches(1); }
             }
             double rr;
-            if ((st = dot_host(c, ws->w, ws->w, &rr)) != CHNS_OK) return st;
+            if ((st = dot_host(c, ws->V, ws->V, &rr)) != CHNS_OK) return st;
             rnorm = std::sqrt(rr);
             {
                 float ms = 0.0f;
@@ -1079,20 +924,6 @@ extern "C" chns_status chns_initial_mu(const chns_mesh* mc, const chns_params* p
 // ---------------------------------------------------------------------------------
 namespace {
 
-template <class TI>
-__global__ void pc_apply_T_kernel(int64_t N, int NF, const TI* __restrict__ inv, const double* __restrict__ v,
-                                  double* __restrict__ z) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    double x[6];
-    for (int j = 0; j < NF; ++j) x[j] = v[(size_t)n * NF + j];
-    for (int i = 0; i < NF; ++i) {
-        double s = 0.0;
-        for (int j = 0; j < NF; ++j) s += (double)inv[((size_t)n * NF + j) * NF + i] * x[j];
-        z[(size_t)n * NF + i] = s;
-    }
-}
-
 // unweighted sum of field f into per-block partials
 __global__ void field_sum_kernel(const double* __restrict__ v, int NF, int f, int64_t N, double* partials) {
     double acc[1] = {0.0};
@@ -1100,13 +931,18 @@ __global__ void field_sum_kernel(const double* __restrict__ v, int NF, int f, in
         acc[0] += v[(size_t)n * NF + f];
     block_reduce_store<1>(acc, partials);
 }
-// sum_n wt[n*NF + f] v[n*NF + f] into per-block partials
+// out = sum_n wt[n*NF + f] v[n*NF + f]: the block that finishes last sums the partials
 __global__ void field_wdot_kernel(const double* __restrict__ wt, const double* __restrict__ v, int NF, int f,
-                                  int64_t N, double* partials) {
+                                  int64_t N, double* partials, unsigned int* counter, double* out) {
     double acc[1] = {0.0};
     for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (int64_t)gridDim.x * blockDim.x)
         acc[0] += wt[(size_t)n * NF + f] * v[(size_t)n * NF + f];
     block_reduce_store<1>(acc, partials);
+    if (!krylov::last_block(counter) || threadIdx.x >= 32) return;
+    double t = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) t += __ldcg(partials + b);
+    t = krylov::warp_sum(t);
+    if (threadIdx.x == 0) out[0] = t;
 }
 // v[n*NF + f] += a * m[n] * sc[0]
 __global__ void field_axpy_mass_kernel(double* __restrict__ v, int NF, int f, int64_t N, const double* __restrict__ m,
@@ -1148,6 +984,7 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
     if (schur && (st = precond_prepare(m, spec, c.s)) != CHNS_OK) return st;
     const int gN = (int)((m->dm.N + 127) / 128);
     const int nbk = c.g < 1024 ? c.g : 1024;
+    const int nbw = std::min(grid_for(m->dm.N), 512);
     chns_stats S;
     std::memset(&S, 0, sizeof(S));
 
@@ -1163,17 +1000,16 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
     // u^T lambda = 0 (GMRES on the singular J^T drifts along its null vector)
     const double inv_vol = 1.0 / m->volume;
     auto add_pmean_T = [&](const double* v, double* y) {
-        { field_wdot_kernel<<<nbk, 256, 0, c.s>>>(ws->Sd, v, NF, D, m->dm.N, m->d_partials); chns_count_launches(1); }
-        { final_reduce_kernel<<<1, 256, 0, c.s>>>(m->d_partials, nbk, 1, ws->sc + 820); chns_count_launches(1); }
-        { field_axpy_mass_kernel<<<c.g, 256, 0, c.s>>>(y, NF, D, m->dm.N, m->d_nmass, ws->sc + 820, inv_vol); chns_count_launches(1); }
+        { field_wdot_kernel<<<nbw, 256, 0, c.s>>>(ws->Sd, v, NF, D, m->dm.N, m->d_partials, ws->counter + 1, ws->sc + SC_MISC + 1); chns_count_launches(1); }
+        { field_axpy_mass_kernel<<<c.g, 256, 0, c.s>>>(y, NF, D, m->dm.N, m->d_nmass, ws->sc + SC_MISC + 1, inv_vol); chns_count_launches(1); }
     };
     // b = P^T g: remove sum(g_p) * m / |Omega| from the pressure part (pin mode 2)
     double* b = ws->R;
     { copy64_kernel<<<c.g, 256, 0, c.s>>>(g, b, c.n); chns_count_launches(1); }
     if (pin == 2) {
         { field_sum_kernel<<<nbk, 256, 0, c.s>>>(g, NF, D, m->dm.N, m->d_partials); chns_count_launches(1); }
-        { final_reduce_kernel<<<1, 256, 0, c.s>>>(m->d_partials, nbk, 1, ws->sc + 800); chns_count_launches(1); }
-        { field_axpy_mass_kernel<<<c.g, 256, 0, c.s>>>(b, NF, D, m->dm.N, m->d_nmass, ws->sc + 800, -1.0 / m->volume); chns_count_launches(1); }
+        { final_reduce_kernel<<<1, 256, 0, c.s>>>(m->d_partials, nbk, 1, ws->sc + SC_MISC); chns_count_launches(1); }
+        { field_axpy_mass_kernel<<<c.g, 256, 0, c.s>>>(b, NF, D, m->dm.N, m->d_nmass, ws->sc + SC_MISC, -1.0 / m->volume); chns_count_launches(1); }
     }
     CHNS_CUDA(cudaGetLastError());
     double bb;
@@ -1188,36 +1024,37 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
         std::vector<double> H((size_t)(mres + 1) * mres), cs(mres), sn(mres), gv(mres + 1), y(mres);
         double rnorm = bnorm;
         int kry = 0;
-        { copy64_kernel<<<c.g, 256, 0, c.s>>>(b, ws->w, c.n); chns_count_launches(1); }
+        { copy64_kernel<<<c.g, 256, 0, c.s>>>(b, ws->V, c.n); chns_count_launches(1); }
+        // slot j + 1 = J^T M^{-T} v_j
+        auto apply_op = [&](int j) -> chns_status {
+            double* w = ws->V + (size_t)(j + 1) * ws->ld;
+            launch_pc_first<true>(m, schur ? 1 : 0, ws->Pinv64, ws->V + (size_t)j * ws->ld, ws->sc + SC_SCALE + j, nullptr, ws->z64, c.s);
+            if (schur && (st = precond_apply(m, spec, ws->z64, PrecondMean(), c.s)) != CHNS_OK) return st;
+            CHNS_CUDA(launch_vjp(m, pc, U_old, U_new, ws->z64, w, nullptr, nullptr, pin, c.s));
+            if (pin == 2) add_pmean_T(ws->z64, w);
+            S.jvp_calls++;
+            return CHNS_OK;
+        };
         while (true) {
             const double beta = rnorm;
-            { axpby_kernel<<<c.g, 256, 0, c.s>>>(1.0 / beta, ws->w, 0.0, ws->V, c.n); chns_count_launches(1); }
+            { set_scalar_kernel<<<1, 1, 0, c.s>>>(ws->sc + SC_SCALE, 1.0 / beta); chns_count_launches(1); }
             std::fill(gv.begin(), gv.end(), 0.0);
             gv[0] = beta;
             int j = 0;
             bool done = false;
+            if ((st = apply_op(0)) != CHNS_OK) return st;
             for (; j < mres && kry < o->max_krylov; ++j, ++kry) {
-                double* Vj = ws->V + (size_t)j * c.n;
-                { pc_apply_T_kernel<double><<<gN, 128, 0, c.s>>>(m->dm.N, NF, ws->Pinv64, Vj, ws->z64); chns_count_launches(1); }
-                if (schur) {
-                    // from a fixed vector, so that one captured graph serves every j
-                    { copy64_kernel<<<c.g, 256, 0, c.s>>>(Vj, ws->SR, c.n); chns_count_launches(1); }
-                    if ((st = precond_apply(m, spec, ws->SR, ws->z64, c.s)) != CHNS_OK) return st;
-                }
-                CHNS_CUDA(launch_vjp(m, pc, U_old, U_new, ws->z64, ws->w, nullptr, nullptr, pin, c.s));
-                if (pin == 2) add_pmean_T(ws->z64, ws->w);
-                S.jvp_calls++;
-                CHNS_CUDA(launch_multidot(m, ws->V, c.n, j + 1, ws->w, c.n, ws->sc, c.s));
-                { gs_update_kernel<<<c.g, 256, 0, c.s>>>(ws->V, c.n, j + 1, ws->sc, ws->w, c.n); chns_count_launches(1); }
-                CHNS_CUDA(launch_multidot(m, ws->V, c.n, j + 1, ws->w, c.n, ws->sc + 256, c.s));
-                { gs_update_kernel<<<c.g, 256, 0, c.s>>>(ws->V, c.n, j + 1, ws->sc + 256, ws->w, c.n); chns_count_launches(1); }
-                CHNS_CUDA(launch_dot(m, ws->w, ws->w, c.n, ws->sc + 512, c.s));
-                double hs[513];
-                CHNS_CUDA(cudaMemcpyAsync(ws->hsc, ws->sc, 513 * sizeof(double), cudaMemcpyDeviceToHost, c.s));
-                CHNS_CUDA(cudaStreamSynchronize(c.s));
-                std::memcpy(hs, ws->hsc, 513 * sizeof(double));
-                const double hn = std::sqrt(hs[512]);
-                for (int i = 0; i <= j; ++i) H[(size_t)i * mres + j] = hs[i] + hs[256 + i];
+                // two full Gram-Schmidt passes, then the next vector's operator queued
+                // before the host waits for this one's column
+                const krylov::Source src{nullptr, nullptr, nullptr, nullptr, 0.0, NF, D};
+                chns_count_launches(krylov::orthogonalise(ws->V, ws->ld, j + 1, src, c.n, ws->sc, HUGE_VAL, ws->hsc, ws->part, ws->counter, c.s));
+                CHNS_CUDA(cudaGetLastError());
+                CHNS_CUDA(cudaEventRecord(ws->ev[10], c.s));
+                if (j + 1 < mres && kry + 1 < o->max_krylov)
+                    if ((st = apply_op(j + 1)) != CHNS_OK) return st;
+                CHNS_CUDA(cudaEventSynchronize(ws->ev[10]));
+                const double hn = std::sqrt(ws->hsc[SC_NA]);
+                for (int i = 0; i <= j; ++i) H[(size_t)i * mres + j] = ws->hsc[i];
                 H[(size_t)(j + 1) * mres + j] = hn;
                 if (!std::isfinite(hn)) { chns_set_error("non-finite Arnoldi vector"); result = CHNS_EBREAKDOWN; break; }
                 for (int i = 0; i < j; ++i) {
@@ -1234,8 +1071,6 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
                 gv[j + 1] = -sn[j] * gv[j];
                 gv[j] = cs[j] * gv[j];
                 rnorm = std::fabs(gv[j + 1]);
-                if (hn > 0.0)
-                    { axpby_kernel<<<c.g, 256, 0, c.s>>>(1.0 / hn, ws->w, 0.0, ws->V + (size_t)(j + 1) * c.n, c.n); chns_count_launches(1); }
                 if (rnorm <= o->krylov_rtol * bnorm || hn == 0.0) {
                     ++j;
                     ++kry;
@@ -1252,19 +1087,20 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
             }
             std::memcpy(ws->hsc, y.data(), k * sizeof(double));
             CHNS_CUDA(cudaMemcpyAsync(ws->sc, ws->hsc, k * sizeof(double), cudaMemcpyHostToDevice, c.s));
-            { combine_kernel<<<c.g, 256, 0, c.s>>>(ws->V, c.n, k, ws->sc, ws->t64, c.n); chns_count_launches(1); }
-            { pc_apply_T_kernel<double><<<gN, 128, 0, c.s>>>(m->dm.N, NF, ws->Pinv64, ws->t64, ws->z64); chns_count_launches(1); }
-            if (schur && (st = precond_apply(m, spec, ws->t64, ws->z64, c.s)) != CHNS_OK) return st;
+            krylov::combine(ws->V, ws->ld, k, ws->sc, ws->sc + SC_SCALE, ws->t64, c.n, c.s);
+            chns_count_launches(1);
+            launch_pc_first<true>(m, schur ? 1 : 0, ws->Pinv64, ws->t64, nullptr, nullptr, ws->z64, c.s);
+            if (schur && (st = precond_apply(m, spec, ws->z64, PrecondMean(), c.s)) != CHNS_OK) return st;
             { axpy_kernel<<<c.g, 256, 0, c.s>>>(1.0, ws->z64, lambda, c.n); chns_count_launches(1); }
             CHNS_CUDA(cudaGetLastError());
             if (done || kry >= o->max_krylov) break;
             // restart: r = b - J^T lambda
-            CHNS_CUDA(launch_vjp(m, pc, U_old, U_new, lambda, ws->w, nullptr, nullptr, pin, c.s));
-            if (pin == 2) add_pmean_T(lambda, ws->w);
+            CHNS_CUDA(launch_vjp(m, pc, U_old, U_new, lambda, ws->V, nullptr, nullptr, pin, c.s));
+            if (pin == 2) add_pmean_T(lambda, ws->V);
             S.jvp_calls++;
-            { axpby_kernel<<<c.g, 256, 0, c.s>>>(1.0, b, -1.0, ws->w, c.n); chns_count_launches(1); }
+            { axpby_kernel<<<c.g, 256, 0, c.s>>>(1.0, b, -1.0, ws->V, c.n); chns_count_launches(1); }
             double rr;
-            if ((st = dot_host(c, ws->w, ws->w, &rr)) != CHNS_OK) return st;
+            if ((st = dot_host(c, ws->V, ws->V, &rr)) != CHNS_OK) return st;
             rnorm = std::sqrt(rr);
             if (rnorm <= o->krylov_rtol * bnorm) break;
         }
@@ -1281,7 +1117,7 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
     if (gCn) { axpby_kernel<<<1, 32, 0, c.s>>>(0.0, gCn, -1.0, gCn, 1); chns_count_launches(1); }
     if (pin == 2) {
         // the normalisation int p^{k+1} = int p^k passes sum(g_p) m / |Omega| to p^k
-        { field_axpy_mass_kernel<<<c.g, 256, 0, c.s>>>(gU_old, NF, D, m->dm.N, m->d_nmass, ws->sc + 800, 1.0 / m->volume); chns_count_launches(1); }
+        { field_axpy_mass_kernel<<<c.g, 256, 0, c.s>>>(gU_old, NF, D, m->dm.N, m->d_nmass, ws->sc + SC_MISC, 1.0 / m->volume); chns_count_launches(1); }
     }
     CHNS_CUDA(cudaGetLastError());
     CHNS_CUDA(cudaStreamSynchronize(c.s));
