@@ -43,7 +43,8 @@ METRIC = "CHNS JÂ·x GDOF/s & % HBM roofline; mixed vs FP64 Newton step time at â
 # reports them as null (stale) until they are captured again.
 # preconditioner of the timed Newton step (chns_solver_opts.pc_type)
 BENCH_PC_TYPE = 1
-KERNEL_SRC_FILES = ("paper_2009_06628_gb300/csrc/element_kernels.cu", "paper_2009_06628_gb300/csrc/pointwise.cuh")
+KERNEL_SRC_FILES = tuple("paper_2009_06628_gb300/csrc/" + f for f in ("element_kernels.cu", "point_physics.cuh", "q1_lanes.cuh",
+                                                                       "replaced_rows.cuh"))
 KERNEL_SRC_SHA = "de8fd3eb9c4ab80e"
 KERNEL_COUNTS = {
     "jvp_fp32": {"flop_per_element": 14769.6, "dram_bytes": 35048192},

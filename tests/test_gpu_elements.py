@@ -72,3 +72,32 @@ def test_element_kernels(chns, dim, kind, level, pin, hi):
     assert abs(float(gc.cpu()[0]) - float(gco)) <= 1e-11 * max(1.0, abs(float(gco)))
     g2, none, _ = chns.vjp(gm, prm, d(Ut), d(Unt), d(w), want_old=False, want_cn=False)
     assert none is None and rel(g2, gno) <= 1e-12
+
+
+@pytest.mark.parametrize("dim,level,hi", [(2, 1, 1.0), (2, 2, 0.7), (2, 3, 1.0), (3, 1, 1.0), (3, 2, 1.4), (2, 6, 1.0)])
+def test_q2_element_kernels(chns, dim, level, hi):
+    """The Q2 kernels at element counts that are no multiple of a warp's 1, 2, 3 or 6 elements, blocks
+    of one and of four warps, and a 4-byte-aligned FP32 output; bars as above."""
+    from oracle import MeshQ2 as OMeshQ2
+    om, gm = OMeshQ2(dim, level, 0.0, hi), chns.MeshQ2(dim, level, 0.0, hi)
+    cfg = synth.config_params("drop3d" if dim == 3 else "drop2d")
+    cfg.update(Fr=1.0, rho_ratio=20.0, eta_ratio=7.0, Cn=0.05)
+    prm, oprm, o = chns.Params.make(**cfg), OParams(**cfg), Oracle(om)
+    rng = np.random.default_rng(6)
+    U = 0.1 * rng.standard_normal((om.N, dim + 3))
+    U[:, dim + 1] = 1.3 * np.sin(3.0 * om.x.sum(axis=1))
+    Un = U + 1e-3 * rng.standard_normal(U.shape)
+    Ut, Unt, x, w = (torch.tensor(a) for a in (U, Un, rng.standard_normal(U.shape), rng.standard_normal(U.shape)))
+    d = lambda t: t.cuda()
+    f = lambda t: t.cuda().float()
+    rel = lambda a, b: float((a.cpu().double() - b).norm() / b.norm())
+    assert rel(chns.residual(gm, prm, d(Ut), d(Unt)), o.residual(oprm, Ut, Unt)) <= 1e-12
+    y = o.jvp(oprm, Ut, Unt, x)
+    assert rel(chns.jvp(gm, prm, d(Ut), d(Unt), d(x)), y) <= 1e-12
+    assert rel(chns.jvp(gm, prm, f(Ut), f(Unt), f(x)), y) <= 1e-5
+    out = torch.empty(U.size + 1, dtype=torch.float32, device="cuda")[1:].view(U.shape)
+    assert rel(chns.jvp(gm, prm, f(Ut), f(Unt), f(x), out=out), y) <= 1e-5
+    gn, go, gc = chns.vjp(gm, prm, d(Ut), d(Unt), d(w))
+    gno, goo, gco = o.vjp(oprm, Ut, Unt, w)
+    assert rel(gn, gno) <= 1e-12 and rel(go, goo) <= 1e-12
+    assert abs(float(gc.cpu()[0]) - float(gco)) <= 1e-11 * max(1.0, abs(float(gco)))
