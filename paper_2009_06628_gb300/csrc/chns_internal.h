@@ -25,6 +25,8 @@ struct DevMesh {
 };
 
 struct SolverWS;  // Newton-Krylov workspace (solver.cu)
+struct MassWS;    // workspace of the mass-matrix solves (mass_cg.cu)
+void chns_mass_ws_free(MassWS* w);
 struct PrecondWS; // preconditioner operators and vectors (precond.cu)
 struct MGHier;    // geometric multigrid hierarchy of the pressure Schur Laplacian (multigrid.cu)
 
@@ -54,9 +56,10 @@ struct chns_mesh {
     double* d_partials = nullptr;
     int64_t n_partials = 0;
     double* h_pinned = nullptr;      // pinned host landing zone for scalar results
-    unsigned int* d_flags = nullptr; // bit 0: a tau radicand was not positive
+    unsigned int* d_flags = nullptr; // word 0, bit 0: a tau radicand was not positive; word 8: blocks done (reductions)
     SolverWS* ws = nullptr;
     MGHier* mg = nullptr;
+    MassWS* mass = nullptr;          // mass-matrix solves (mass_cg.cu)
     PrecondWS* pre = nullptr;        // assembled operators of the preconditioners (precond.cu)
     // scatter strategy of the element kernels (0 atomics, 1 colouring, 2 warp-aggregated)
     int32_t scatter = 0;
@@ -103,8 +106,6 @@ cudaError_t launch_energy(const chns_mesh* m, const PhysConst& pc, const double*
 // deterministic FP64 reductions into device scalars (solver.cu uses them)
 cudaError_t launch_dot(const chns_mesh* m, const double* a, const double* b, int64_t n, double* out_dev,
                        cudaStream_t s);
-cudaError_t launch_multidot(const chns_mesh* m, const double* V, int64_t ld, int k, const double* w, int64_t n,
-                            double* out_dev, cudaStream_t s);
 
 // ---------------------------------------------------------------------------------
 // Transfer between the Q1 spaces of two meshes of the same domain (multigrid.cu):

@@ -317,6 +317,7 @@ void precond_free(PrecondWS* p);         // precond.cu
 extern "C" void chns_mesh_destroy(chns_mesh* m) {
     if (!m) return;
     precond_free(m->pre);
+    chns_mass_ws_free(m->mass);
     if (m->ws) chns_solver_ws_free(m->ws);
     if (m->mg) chns_mg_free(m->mg);
     cudaFree(m->d_e2n);

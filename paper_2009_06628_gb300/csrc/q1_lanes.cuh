@@ -42,6 +42,9 @@ template <> struct Lanes<float2> {
     using XD = float;
 };
 
+// 2^k, |k| < 1022
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+
 __device__ __forceinline__ double shx(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
 __device__ __forceinline__ float shx(float v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
 __device__ __forceinline__ float2 shx(float2 v, int m) {

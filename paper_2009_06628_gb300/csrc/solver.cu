@@ -9,8 +9,7 @@
 // J dU = -R.  Gram-Schmidt (including the decision to re-orthogonalise) and the next
 // Arnoldi vector stay on the device; the Hessenberg column goes to the host for the
 // Givens update, and that read-back overlaps the next vector's operator application,
-// which is queued before the host waits.  Also: the consistent initial chemical
-// potential by CG.
+// which is queued before the host waits.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -196,37 +195,6 @@ int grid_for(int64_t n) {
 }
 
 // ---------------- block-Jacobi preconditioner ----------------
-constexpr double GPc = 0.78867513459481288225, GMc = 0.21132486540518711775;
-
-template <int D, class T>
-struct PB {
-    T N, dN[D], d2N[D == 2 ? 1 : 3];
-};
-template <int D, class T>
-__device__ __forceinline__ PB<D, T> pbasis(int a, int q, T inv_h) {
-    T f[D], s[D];
-    for (int k = 0; k < D; ++k) {
-        f[k] = (((a >> k) & 1) == ((q >> k) & 1)) ? T(GPc) : T(GMc);
-        s[k] = ((a >> k) & 1) ? inv_h : -inv_h;
-    }
-    PB<D, T> b;
-    if constexpr (D == 2) {
-        b.N = f[0] * f[1];
-        b.dN[0] = s[0] * f[1];
-        b.dN[1] = f[0] * s[1];
-        b.d2N[0] = s[0] * s[1];
-    } else {
-        b.N = f[0] * f[1] * f[2];
-        b.dN[0] = s[0] * f[1] * f[2];
-        b.dN[1] = f[0] * s[1] * f[2];
-        b.dN[2] = f[0] * f[1] * s[2];
-        b.d2N[0] = s[0] * s[1] * f[2];
-        b.d2N[1] = s[0] * f[1] * s[2];
-        b.d2N[2] = f[0] * s[1] * s[2];
-    }
-    return b;
-}
-
 // Replace Dirichlet / pin rows by identity rows and invert every block (Gauss-Jordan
 // with partial pivoting in FP64).
 template <class TB, class TI>
@@ -349,70 +317,6 @@ void launch_pc_first(const chns_mesh* m, int mask, const TI* inv, const double* 
 }
 __global__ void set_scalar_kernel(double* p, double v) { *p = v; }
 
-// ---------------- initial chemical potential (mass-matrix CG) ----------------
-// b_a = sum_q |J| (N_a psi'(phi_q) + Cn^2 grad N_a . grad phi_q)  and  y = M x, with the
-// consistent Q1 mass matrix; hanging corners via their parents.
-template <int D, int MODE>
-__global__ void mu_kernel(DevMesh m, double Cn2, const double* __restrict__ U, const double* __restrict__ x,
-                          double* __restrict__ y) {
-    constexpr int NC = 1 << D, NF = D + 3;
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= m.E) return;
-    const double h = ldexp(m.hi - m.lo, -(int)m.level[e]);
-    const double inv_h = 1.0 / h, detJ = (D == 2) ? 0.25 * h * h : 0.125 * h * h * h;
-    int par[NC][4], np[NC];
-    double u[NC];
-    for (int a = 0; a < NC; ++a) {
-        const int ent = m.e2n[e * NC + a];
-        if (ent >= 0) {
-            np[a] = 1;
-            par[a][0] = ent;
-        } else {
-            const int4 hp = reinterpret_cast<const int4*>(m.hang)[-ent - 1];
-            par[a][0] = hp.x;
-            par[a][1] = hp.y;
-            par[a][2] = hp.z;
-            par[a][3] = hp.w;
-            np[a] = hp.z < 0 ? 2 : 4;
-        }
-        const double w = np[a] == 1 ? 1.0 : (np[a] == 2 ? 0.5 : 0.25);
-        double s = 0.0;
-        for (int j = 0; j < np[a]; ++j)
-            s += w * (MODE == 0 ? U[(size_t)par[a][j] * NF + D + 1] : x[par[a][j]]);
-        u[a] = s;
-    }
-    double r[NC];
-    for (int a = 0; a < NC; ++a) r[a] = 0.0;
-    for (int q = 0; q < NC; ++q) {
-        double val = 0.0, grad[D];
-        for (int k = 0; k < D; ++k) grad[k] = 0.0;
-        PB<D, double> B[NC];
-        for (int a = 0; a < NC; ++a) {
-            B[a] = pbasis<D, double>(a, q, inv_h);
-            val += B[a].N * u[a];
-            for (int k = 0; k < D; ++k) grad[k] += B[a].dN[k] * u[a];
-        }
-        for (int a = 0; a < NC; ++a) {
-            double t;
-            if (MODE == 0) {
-                t = B[a].N * (val * val * val - val);
-                for (int k = 0; k < D; ++k) t += Cn2 * B[a].dN[k] * grad[k];
-            } else {
-                t = B[a].N * val;
-            }
-            r[a] += detJ * t;
-        }
-    }
-    for (int a = 0; a < NC; ++a) {
-        const double w = np[a] == 1 ? 1.0 : (np[a] == 2 ? 0.5 : 0.25);
-        for (int j = 0; j < np[a]; ++j) atomicAdd(y + par[a][j], w * r[a]);
-    }
-}
-
-__global__ void insert_mu_kernel(const double* __restrict__ in, int NF, int f, int64_t N, double* __restrict__ U) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) U[(size_t)n * NF + f] = in[n];
-}
 // sum_n m_n v[n*NF + f] into per-block partials
 template <class T>
 __global__ void field_mass_kernel(const double* __restrict__ m, const T* __restrict__ v, int NF, int f,
@@ -443,16 +347,6 @@ __global__ void field_shift_kernel(double* __restrict__ v, int NF, int f, int64_
     for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (int64_t)gridDim.x * blockDim.x)
         v[(size_t)n * NF + f] -= s;
 }
-__global__ void fill_kernel(double* __restrict__ x, double v, int64_t n) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        x[i] = v;
-}
-__global__ void jacobi_kernel(const double* __restrict__ d, const double* __restrict__ r, double* __restrict__ z,
-                              int64_t N) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) z[n] = r[n] / d[n];
-}
-
 struct Ctx {
     chns_mesh* m;
     SolverWS* ws;
@@ -842,80 +736,6 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
     return result;
 }
 
-extern "C" chns_status chns_initial_mu(const chns_mesh* mc, const chns_params* p, double* U, void* stream) {
-    if (chns_require_q1(mc, "chns_initial_mu") != CHNS_OK) return CHNS_EINVAL;
-    chns_mesh* m = const_cast<chns_mesh*>(mc);
-    PhysConst pc;
-    chns_status st = chns_check_params(mc, p, &pc);
-    if (st != CHNS_OK) return st;
-    if (!U) { chns_set_error("null argument"); return CHNS_EINVAL; }
-    if ((st = ensure_ws(m, m->ws ? m->ws->restart : 1)) != CHNS_OK) return st;
-    SolverWS* ws = m->ws;
-    const int64_t N = m->dm.N;
-    Ctx c{m, ws, (cudaStream_t)stream, N, grid_for(N)};
-    const int D = m->dm.dim, NF = m->dm.nf;
-    const int gE = (int)((m->dm.E + 127) / 128), gN = (int)((N + 255) / 256);
-    // work vectors (each N doubles) carved from the Krylov workspace
-    double* b = ws->w;
-    double* x = ws->R;
-    double* r = ws->dU;
-    double* z = ws->z64;
-    double* q = ws->t64;
-    double* dg = ws->V;
-    double* pvec = ws->V + N;
-    const double Cn2 = p->Cn * p->Cn;
-    cudaError_t e = cudaMemsetAsync(b, 0, N * sizeof(double), c.s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dg, 0, N * sizeof(double), c.s);
-    if (e != cudaSuccess) return chns_cuda_status(e, "cudaMemsetAsync");
-    if (D == 2) {
-        { mu_kernel<2, 0><<<gE, 128, 0, c.s>>>(m->dm, Cn2, U, nullptr, b); chns_count_launches(1); }
-    } else {
-        { mu_kernel<3, 0><<<gE, 128, 0, c.s>>>(m->dm, Cn2, U, nullptr, b); chns_count_launches(1); }
-    }
-    // Jacobi scaling by the row sums of M (the integral of each basis function, > 0)
-    { fill_kernel<<<c.g, 256, 0, c.s>>>(q, 1.0, N); chns_count_launches(1); }
-    if (D == 2)
-        { mu_kernel<2, 1><<<gE, 128, 0, c.s>>>(m->dm, Cn2, U, q, dg); chns_count_launches(1); }
-    else
-        { mu_kernel<3, 1><<<gE, 128, 0, c.s>>>(m->dm, Cn2, U, q, dg); chns_count_launches(1); }
-    CHNS_CUDA(cudaGetLastError());
-    // CG from x = 0
-    CHNS_CUDA(cudaMemsetAsync(x, 0, N * sizeof(double), c.s));
-    { copy64_kernel<<<c.g, 256, 0, c.s>>>(b, r, N); chns_count_launches(1); }
-    { jacobi_kernel<<<gN, 256, 0, c.s>>>(dg, r, z, N); chns_count_launches(1); }
-    { copy64_kernel<<<c.g, 256, 0, c.s>>>(z, pvec, N); chns_count_launches(1); }
-    double rz, bb;
-    if ((st = dot_host(c, r, z, &rz)) != CHNS_OK) return st;
-    if ((st = dot_host(c, b, b, &bb)) != CHNS_OK) return st;
-    const double tol = 1e-14 * std::sqrt(bb);
-    int it = 0;
-    for (; it < 1000 && bb > 0.0; ++it) {
-        CHNS_CUDA(cudaMemsetAsync(q, 0, N * sizeof(double), c.s));
-        if (D == 2)
-            { mu_kernel<2, 1><<<gE, 128, 0, c.s>>>(m->dm, Cn2, U, pvec, q); chns_count_launches(1); }
-        else
-            { mu_kernel<3, 1><<<gE, 128, 0, c.s>>>(m->dm, Cn2, U, pvec, q); chns_count_launches(1); }
-        double pq, rr;
-        if ((st = dot_host(c, pvec, q, &pq)) != CHNS_OK) return st;
-        const double alpha = rz / pq;
-        { axpy_kernel<<<c.g, 256, 0, c.s>>>(alpha, pvec, x, N); chns_count_launches(1); }
-        { axpy_kernel<<<c.g, 256, 0, c.s>>>(-alpha, q, r, N); chns_count_launches(1); }
-        if ((st = dot_host(c, r, r, &rr)) != CHNS_OK) return st;
-        if (!std::isfinite(rr)) { chns_set_error("non-finite CG residual"); return CHNS_ENAN; }
-        if (std::sqrt(rr) <= tol) break;
-        { jacobi_kernel<<<gN, 256, 0, c.s>>>(dg, r, z, N); chns_count_launches(1); }
-        double rz2;
-        if ((st = dot_host(c, r, z, &rz2)) != CHNS_OK) return st;
-        { axpby_kernel<<<c.g, 256, 0, c.s>>>(1.0, z, rz2 / rz, pvec, N); chns_count_launches(1); }
-        rz = rz2;
-    }
-    { insert_mu_kernel<<<gN, 256, 0, c.s>>>(x, NF, D + 2, N, U); chns_count_launches(1); }
-    CHNS_CUDA(cudaGetLastError());
-    CHNS_CUDA(cudaStreamSynchronize(c.s));
-    if (it >= 1000) { chns_set_error("mass-matrix CG did not converge"); return CHNS_ENOCONV; }
-    return CHNS_OK;
-}
-
 // ---------------------------------------------------------------------------------
 // Adjoint of one implicit step (reverse mode through Section 3.4's solve): with
 // R(U^k, U^{k+1}; Cn) = 0, a cotangent g of U^{k+1} gives J^T lambda = P^T g
@@ -1124,61 +944,4 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
     S.reason = result;
     if (stats) *stats = S;
     return result;
-}
-
-// M x = rhs with the consistent Q1 mass matrix (hanging constraints included), by
-// Jacobi-preconditioned CG to a relative residual of 1e-14.  Used by the reverse mode
-// of mu^0 (M is symmetric, so its adjoint is the same solve).
-extern "C" chns_status chns_mass_solve(const chns_mesh* mc, const double* rhs, double* x, void* stream) {
-    if (chns_require_q1(mc, "chns_mass_solve") != CHNS_OK) return CHNS_EINVAL;
-    chns_mesh* m = const_cast<chns_mesh*>(mc);
-    if (!m || !rhs || !x) { chns_set_error("null argument"); return CHNS_EINVAL; }
-    chns_status st = ensure_ws(m, m->ws ? m->ws->restart : 1);
-    if (st != CHNS_OK) return st;
-    SolverWS* ws = m->ws;
-    const int64_t N = m->dm.N;
-    const int D = m->dm.dim;
-    Ctx c{m, ws, (cudaStream_t)stream, N, grid_for(N)};
-    const int gE = (int)((m->dm.E + 127) / 128), gN = (int)((N + 255) / 256);
-    double* r = ws->dU;
-    double* z = ws->z64;
-    double* q = ws->t64;
-    double* dg = ws->V;
-    double* pvec = ws->V + N;
-    CHNS_CUDA(cudaMemsetAsync(dg, 0, N * sizeof(double), c.s));
-    { fill_kernel<<<c.g, 256, 0, c.s>>>(q, 1.0, N); chns_count_launches(1); }
-    if (D == 2) { mu_kernel<2, 1><<<gE, 128, 0, c.s>>>(m->dm, 0.0, nullptr, q, dg); chns_count_launches(1); }
-    else { mu_kernel<3, 1><<<gE, 128, 0, c.s>>>(m->dm, 0.0, nullptr, q, dg); chns_count_launches(1); }
-    CHNS_CUDA(cudaMemsetAsync(x, 0, N * sizeof(double), c.s));
-    { copy64_kernel<<<c.g, 256, 0, c.s>>>(rhs, r, N); chns_count_launches(1); }
-    { jacobi_kernel<<<gN, 256, 0, c.s>>>(dg, r, z, N); chns_count_launches(1); }
-    { copy64_kernel<<<c.g, 256, 0, c.s>>>(z, pvec, N); chns_count_launches(1); }
-    CHNS_CUDA(cudaGetLastError());
-    double rz, bb;
-    if ((st = dot_host(c, r, z, &rz)) != CHNS_OK) return st;
-    if ((st = dot_host(c, rhs, rhs, &bb)) != CHNS_OK) return st;
-    const double tol = 1e-14 * std::sqrt(bb);
-    int it = 0;
-    for (; it < 1000 && bb > 0.0; ++it) {
-        CHNS_CUDA(cudaMemsetAsync(q, 0, N * sizeof(double), c.s));
-        if (D == 2) { mu_kernel<2, 1><<<gE, 128, 0, c.s>>>(m->dm, 0.0, nullptr, pvec, q); chns_count_launches(1); }
-        else { mu_kernel<3, 1><<<gE, 128, 0, c.s>>>(m->dm, 0.0, nullptr, pvec, q); chns_count_launches(1); }
-        double pq, rr;
-        if ((st = dot_host(c, pvec, q, &pq)) != CHNS_OK) return st;
-        const double alpha = rz / pq;
-        { axpy_kernel<<<c.g, 256, 0, c.s>>>(alpha, pvec, x, N); chns_count_launches(1); }
-        { axpy_kernel<<<c.g, 256, 0, c.s>>>(-alpha, q, r, N); chns_count_launches(1); }
-        if ((st = dot_host(c, r, r, &rr)) != CHNS_OK) return st;
-        if (!std::isfinite(rr)) { chns_set_error("non-finite CG residual"); return CHNS_ENAN; }
-        if (std::sqrt(rr) <= tol) break;
-        { jacobi_kernel<<<gN, 256, 0, c.s>>>(dg, r, z, N); chns_count_launches(1); }
-        double rz2;
-        if ((st = dot_host(c, r, z, &rz2)) != CHNS_OK) return st;
-        { axpby_kernel<<<c.g, 256, 0, c.s>>>(1.0, z, rz2 / rz, pvec, N); chns_count_launches(1); }
-        rz = rz2;
-    }
-    CHNS_CUDA(cudaGetLastError());
-    CHNS_CUDA(cudaStreamSynchronize(c.s));
-    if (it >= 1000) { chns_set_error("mass-matrix CG did not converge"); return CHNS_ENOCONV; }
-    return CHNS_OK;
 }
