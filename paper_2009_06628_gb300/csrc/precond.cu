@@ -462,13 +462,6 @@ __global__ void __launch_bounds__(256) residual_kernel(Sell S, const float* __re
     const float y = row_dot<LPR>(S, val, n, [&](int q) { return __ldg(x + q); });
     if (store) t[n] = b[n] - y;
 }
-template <class TO>
-__global__ void store_kernel(int64_t N, int NF, int f, const float* __restrict__ x, TO* __restrict__ z, PrecondMean mean) {
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const float v = n < N ? x[n] : 0.0f;
-    if (n < N) z[(size_t)n * NF + f] = (TO)v;
-    if (mean.out) mean_add(mean, n < N ? mean.nmass[n] * (double)v : 0.0);
-}
 // r = base + c A (x .* m): the right-hand side of a Chebyshev solve (base, m may be null)
 template <int LPR>
 __global__ void __launch_bounds__(256) rhs_kernel(Sell S, const float* __restrict__ val, const float* __restrict__ x,
@@ -579,19 +572,96 @@ __device__ void tail_cheb_l(const TailLevel& L, const float* in, float* out) {
         dn = const_cast<float*>(tmp);
     }
 }
+// The same with everything but d in registers: a thread holds R rows of at most W entries (columns
+// as 16-bit numbers), a slice of rows per warp, G entries at a time.  A step is then one gather from
+// shared memory per entry and a barrier; from L1 it was three loads.
+// 1,089 rows of 9 (2D), degree 16: the kernel 34 -> 18 us (and a second one of 4.6 us, which stored the
+// result, went); 729 rows of 21 (3D): 17.2 -> 12.5 us; a V-cycle over 45,000 rows: 2 % of the
+// application.  Half the threads with twice the rows: 17.1, 13.7 us and 2 % slower.
+constexpr int TAIL_ROWS = 2 * TAIL_THREADS;
+template <int R, int W, int G, bool ADD>
+__device__ void tail_cheb_r(const TailLevel& L, const float* in, float* out, float (*sd)[TAIL_ROWS]) {
+    const ChebCoef* cf = L.cf;
+    const float it = __ldg(&cf->inv_theta);
+    const int lane = threadIdx.x & 31, N = (int)L.S.N;
+    float v[R][W], di[R], r[R], x[R], d[R];
+    unsigned int c[R][W / 2];
+    int w[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const int s = (threadIdx.x >> 5) + i * (TAIL_THREADS / 32), n = s * 32 + lane;
+        const int64_t o0 = s < L.S.ns ? __ldg(L.S.off + s) : 0;
+        w[i] = s < L.S.ns ? (int)((__ldg(L.S.off + s + 1) - o0) >> 5) : 0;
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            const bool has = j < w[i] && n < N;
+            v[i][j] = has ? __ldg(L.val + o0 + lane + 32 * j) : 0.0f;
+            const unsigned int q = has ? (unsigned int)__ldg(L.S.col + o0 + lane + 32 * j) : 0u;
+            c[i][j / 2] = j & 1 ? c[i][j / 2] | q << 16 : q;
+        }
+        di[i] = n < N ? __ldg(L.dinv + n) : 0.0f;
+        r[i] = n < N ? in[n] : 0.0f;
+        d[i] = it * di[i] * r[i];
+        x[i] = 0.0f;
+        sd[0][n] = d[i];
+    }
+    float c1 = __ldg(cf->c1), c2 = __ldg(cf->c2);
+    __syncthreads();
+    for (int k = 0; k + 1 < L.deg; ++k) {
+        const bool last = k + 2 == L.deg;
+        const float* ds = sd[k & 1];
+        const float n1 = last ? 0.0f : __ldg(cf->c1 + k + 1), n2 = last ? 0.0f : __ldg(cf->c2 + k + 1);
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const int n = (int)(threadIdx.x & ~31u) + i * TAIL_THREADS + lane;
+            float y = 0.0f;
+#pragma unroll
+            for (int g = 0; g < W; g += G) {
+                if (g >= w[i]) break;
+#pragma unroll
+                for (int j = g / 2; j <= (g + G - 1) / 2; ++j) asm volatile("" : "+r"(c[i][j]));   // stays packed
+#pragma unroll
+                for (int j = g; j < g + G; ++j)
+                    y = fmaf(v[i][j], ds[j & 1 ? c[i][j / 2] >> 16 : c[i][j / 2] & 0xffffu], y);
+            }
+            r[i] -= y;
+            x[i] += d[i];
+            d[i] = c1 * d[i] + c2 * di[i] * r[i];
+            if (!last) sd[(k + 1) & 1][n] = d[i];
+            else if (n < N) out[n] = ADD ? out[n] + (x[i] + d[i]) : x[i] + d[i];
+        }
+        c1 = n1;
+        c2 = n2;
+        __syncthreads();
+    }
+}
+// The register form where it fits and is long enough to pay for its loads; else from L1, eight lanes
+// per row where that leaves one round.
 template <bool ADD>
-__device__ void tail_cheb(const TailLevel& L, const float* in, float* out) {
+__device__ void tail_cheb(const TailLevel& L, const float* in, float* out, float (*sd)[TAIL_ROWS]) {
+    if (L.deg > 4 && L.S.N <= TAIL_ROWS) {
+        int w = 0;
+        for (int64_t s = threadIdx.x; s < L.S.ns; s += TAIL_THREADS)
+            w = max(w, (int)((__ldg(L.S.off + s + 1) - __ldg(L.S.off + s)) >> 5));
+        const bool w12 = __syncthreads_and(w <= 12), w24 = __syncthreads_and(w <= 24);
+        if (L.S.N <= TAIL_THREADS && w24) return tail_cheb_r<1, 24, 3, ADD>(L, in, out, sd);
+        if (w12) return tail_cheb_r<2, 12, 3, ADD>(L, in, out, sd);
+    }
     if (L.S.N * 8 <= TAIL_THREADS) tail_cheb_l<8, ADD>(L, in, out);
     else tail_cheb_l<1, ADD>(L, in, out);
 }
-// V-cycle over the block's levels (one level: its polynomial): L[0].b -> L[0].x
-__global__ void __launch_bounds__(TAIL_THREADS) tail_kernel(const Tail* __restrict__ tp) {
+// V-cycle over the block's levels (one level: its polynomial): L[0].b -> L[0].x, and to the strided
+// field f of z (z not null), with its mean
+template <class TO>
+__global__ void __launch_bounds__(TAIL_THREADS) tail_kernel(const Tail* __restrict__ tp, TO* __restrict__ z, int NF, int f,
+                                                            PrecondMean mean) {
+    __shared__ float sd[2][TAIL_ROWS];
     const Tail& T = *tp;
     const int64_t t0 = threadIdx.x, nt = TAIL_THREADS;
     for (int l = 0; l + 1 < T.n; ++l) {
         const TailLevel& L = T.L[l];
         const TailLevel& C = T.L[l + 1];
-        tail_cheb<false>(L, L.b, L.x);
+        tail_cheb<false>(L, L.b, L.x, sd);
         for (int64_t n = t0; n < L.S.N; n += nt)
             L.t[n] = L.b[n] - row_dot<1>(L.S, L.val, n, [&](int q) { return L.x[q]; });
         __syncthreads();
@@ -599,7 +669,7 @@ __global__ void __launch_bounds__(TAIL_THREADS) tail_kernel(const Tail* __restri
         __syncthreads();
     }
     const TailLevel& B = T.L[T.n - 1];
-    tail_cheb<false>(B, B.b, B.x);
+    tail_cheb<false>(B, B.b, B.x, sd);
     for (int l = T.n - 2; l >= 0; --l) {
         const TailLevel& L = T.L[l];
         const TailLevel& C = T.L[l + 1];
@@ -608,7 +678,34 @@ __global__ void __launch_bounds__(TAIL_THREADS) tail_kernel(const Tail* __restri
         for (int64_t n = t0; n < L.S.N; n += nt)
             L.b[n] -= row_dot<1>(L.S, L.val, n, [&](int q) { return L.x[q]; });
         __syncthreads();
-        tail_cheb<true>(L, L.b, L.x);
+        tail_cheb<true>(L, L.b, L.x, sd);
+    }
+    if (!z) return;
+    const TailLevel& F = T.L[0];
+    double acc = 0.0;
+    for (int64_t n = t0; n < F.S.N; n += nt) {
+        const float v = F.x[n];
+        z[(size_t)n * NF + f] = (TO)v;
+        if (mean.out) acc = fma(__ldg(mean.nmass + n), (double)v, acc);
+    }
+    if (!mean.out) return;
+    // four warps, one per scheduler, then one
+    double* sh = reinterpret_cast<double*>(sd);
+    sh[t0] = acc;
+    __syncthreads();
+    if (t0 < 128) {
+        acc = 0.0;
+#pragma unroll
+        for (int q = 0; q < TAIL_THREADS / 128; ++q) acc += sh[t0 + 128 * q];
+    }
+    __syncthreads();
+    if (t0 < 128) sh[t0] = acc;
+    __syncthreads();
+    if (t0 < 32) {
+        acc = (sh[t0] + sh[t0 + 32]) + (sh[t0 + 64] + sh[t0 + 96]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (t0 == 0) mean.out[0] = acc;
     }
 }
 template <class T>
@@ -874,7 +971,6 @@ cudaError_t vcycle(chns_mesh* m, const PrecondSpec& spec, TO* z, int NF, int f, 
                    int* nk) {
     PrecondWS* p = m->pre;
     const int from = p->tail_from;
-    Level& L0 = p->lv[0];
     for (int l = 0; l < from; ++l) {
         Level& L = p->lv[(size_t)l];
         *nk += smooth<float>(L, p->cf + l, spec.degree, nullptr, L.x, 1, 0, PrecondMean(), st);
@@ -883,7 +979,8 @@ cudaError_t vcycle(chns_mesh* m, const PrecondSpec& spec, TO* z, int NF, int f, 
         if (e != cudaSuccess) return e;
         *nk += 2;
     }
-    tail_kernel<<<1, TAIL_THREADS, 0, st>>>(p->tail);
+    const bool all = from == 0;   // every level runs in the one block
+    tail_kernel<TO><<<1, TAIL_THREADS, 0, st>>>(p->tail, all ? z : nullptr, NF, f, all ? mean : PrecondMean());
     ++*nk;
     for (int l = from - 1; l >= 0; --l) {
         Level& L = p->lv[(size_t)l];
@@ -894,10 +991,6 @@ cudaError_t vcycle(chns_mesh* m, const PrecondSpec& spec, TO* z, int NF, int f, 
         *nk += l == 0 ? smooth<TO>(L, p->cf, spec.degree, L.x, z, NF, f, mean, st)
                       : smooth<float>(L, p->cf + l, spec.degree, L.x, L.x, 1, 0, PrecondMean(), st);
     }
-    if (from == 0) {
-        store_kernel<TO><<<blocks_for(L0.dm.N), 256, 0, st>>>(L0.dm.N, NF, f, L0.x, z, mean);
-        ++*nk;
-    }
     return cudaGetLastError();
 }
 template <class TO>
@@ -906,9 +999,8 @@ cudaError_t polynomial(chns_mesh* m, const PrecondSpec& spec, TO* z, int NF, int
     PrecondWS* p = m->pre;
     Level& L = p->lv[0];
     if (p->tail_from == 0) {
-        tail_kernel<<<1, TAIL_THREADS, 0, st>>>(p->tail);
-        store_kernel<TO><<<blocks_for(L.dm.N), 256, 0, st>>>(L.dm.N, NF, f, L.x, z, mean);
-        *nk += 2;
+        tail_kernel<TO><<<1, TAIL_THREADS, 0, st>>>(p->tail, z, NF, f, mean);
+        ++*nk;
         return cudaGetLastError();
     }
     *nk += smooth<TO>(L, p->cf, spec.degree, nullptr, z, NF, f, mean, st);
