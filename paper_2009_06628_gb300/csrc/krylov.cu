@@ -18,6 +18,7 @@
 //   n = 1.65 M, k = 1..30: dots 3.3 us per column + 24 us (w formed, 4 us of reduction), update
 //   2.7 us per column + 10 us; all of an Arnoldi step's vector work 181 -> 136 us, and without the
 //   33 us of the normalising, scaling and mean passes that it takes in.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -33,6 +34,30 @@ __device__ __forceinline__ double formed(const Source& s, int64_t i, double mean
     const double y = s.yf ? (double)s.yf[i] : s.yd[i];
     const double w = s.S[i] * y;
     return s.mean && (int)((uint32_t)i % (uint32_t)s.NF) == s.f ? w + mean : w;   // n < 2^32
+}
+
+// sums of KP numbers (a power of two, at most 32) over the warp: halved over the lanes, then one
+// number per lane group.  Sum number `returned` ends up in acc[0].
+template <int KP>
+__device__ __forceinline__ int warp_sums(double* acc, int lane) {
+    int base = 0, cnt = KP;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        if (cnt > 1) {
+            cnt /= 2;
+            const bool up = lane & o;
+#pragma unroll
+            for (int t = 0; t < KP / 2; ++t) {
+                if (t >= cnt) break;
+                const double keep = up ? acc[cnt + t] : acc[t], give = up ? acc[t] : acc[cnt + t];
+                acc[t] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+            base += up ? cnt : 0;
+        } else {
+            acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+        }
+    }
+    return base;
 }
 
 // h = s .* (V^T w) for K <= 32 columns starting at V, and |w|^2 (nrm not null).  With a source w is
@@ -75,26 +100,7 @@ dots_kernel(const double* __restrict__ V, int64_t ld, Source src, double* w, int
 #pragma unroll
         for (int j = 0; j < K; ++j) acc[j] = fma(V[(size_t)j * ld + i], x, acc[j]);
     }
-    // halve the numbers over the warp's lanes, then one number per lane group
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int base = 0, cnt = KP;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        if (cnt > 1) {
-            cnt /= 2;
-            const bool up = lane & o;
-#pragma unroll
-            for (int t = 0; t < KP / 2; ++t) {
-                if (t >= cnt) break;
-                const double keep = up ? acc[cnt + t] : acc[t], give = up ? acc[t] : acc[cnt + t];
-                acc[t] = keep + __shfl_xor_sync(full, give, o);
-            }
-            base += up ? cnt : 0;
-        } else {
-            acc[0] += __shfl_xor_sync(full, acc[0], o);
-        }
-    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, base = warp_sums<KP>(acc, lane);
     __shared__ double sh[T / 32][KP + 1];
     __shared__ double fin[T];
     sh[warp][base] = acc[0];   // lanes that share a number hold the same sum
@@ -207,6 +213,176 @@ __global__ void __launch_bounds__(T, 4) update_kernel(const double* __restrict__
     __threadfence_system();
 }
 
+// Short vectors: the whole Arnoldi step in one cluster of 16 blocks, w in registers.  Sums cross the
+// blocks through distributed shared memory and two cluster barriers per pass, where the kernels above
+// are four launches (six and more from 33 columns on) of 6 to 10 us that mostly wait.
+//   n = 5,445 (2D), 20 columns on average: 35 -> 20 us per Arnoldi step; n = 4,374 (3D), 60 columns
+//   and two passes: 26 us.  FP64 bound: 2 n k FMAs per pass on 16 SMs, 0.03 ns each.
+namespace cg = cooperative_groups;
+constexpr int CB = 16, CT = 256, CW = CT / 32, CP = 4;
+constexpr int64_t CLUSTER_N = (int64_t)CB * CT * CP * 2;
+
+__device__ __forceinline__ double2 load2(const double* p, int64_t i, int64_t n) {
+    return i + 1 < n ? *reinterpret_cast<const double2*>(p + i) : make_double2(p[i], 0.0);
+}
+__global__ void __launch_bounds__(CT, 1) cluster_kernel(double* V, int64_t ld, int k, Source src, int64_t n, double* __restrict__ sc,
+                                                        double thr, double* host) {
+    __shared__ double part[CW][257];   // sums of each warp: column j, then |w|^2
+    __shared__ double blk[2][257];     // of the block, per pass; read by the whole cluster
+    __shared__ double fin[4][64], c[256], nrm[2][CW], bn[2];
+    cg::cluster_group cl = cg::this_cluster();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t pairs = (n + 1) / 2, q0 = (int64_t)blockIdx.x * CT + threadIdx.x;
+    const bool busy = q0 - lane < pairs;   // the warp has entries at all (P = 0 then for some lanes)
+    double* w = V + (size_t)k * ld;
+    double2 x[CP];
+    int64_t at[CP];
+    const double mean = src.mean ? src.a * src.mean[0] : 0.0;
+    double before = 0.0;
+#pragma unroll
+    for (int p = 0; p < CP; ++p) {
+        const int64_t q = q0 + (int64_t)p * (CB * CT);
+        at[p] = q < pairs ? 2 * q : -1;
+        x[p] = make_double2(0.0, 0.0);
+        if (at[p] >= 0) {
+            if (src.yf || src.yd) x[p] = make_double2(formed(src, at[p], mean), at[p] + 1 < n ? formed(src, at[p] + 1, mean) : 0.0);
+            else x[p] = load2(w, at[p], n);
+        }
+        before = fma(x[p].y, x[p].y, fma(x[p].x, x[p].x, before));
+    }
+    double tot = 0.0;
+    for (int pass = 0; pass < 2; ++pass) {
+        if (busy) {
+            for (int j0 = 0; j0 < k; j0 += 8) {
+                double acc[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) acc[t] = 0.0;
+#pragma unroll
+                for (int p = 0; p < CP; ++p) {
+                    if (at[p] < 0) break;
+                    double2 v[8];
+#pragma unroll
+                    for (int t = 0; t < 8; ++t)
+                        if (j0 + t < k) v[t] = load2(V + (size_t)(j0 + t) * ld, at[p], n);
+#pragma unroll
+                    for (int t = 0; t < 8; ++t)
+                        if (j0 + t < k) acc[t] = fma(v[t].y, x[p].y, fma(v[t].x, x[p].x, acc[t]));
+                }
+                __syncwarp();
+                const int j = j0 + warp_sums<8>(acc, lane);
+                if (j < k) part[warp][j] = acc[0];   // lanes that share a number hold the same sum
+            }
+            if (pass == 0) {
+                before = warp_sum(before);
+                if (lane == 0) part[warp][k] = before;
+            }
+        } else {
+            for (int j = lane; j <= k; j += 32) part[warp][j] = 0.0;
+        }
+        __syncthreads();
+        const int cols = k + (pass == 0 ? 1 : 0);
+        for (int j = threadIdx.x; j < cols; j += CT) {
+            double s = 0.0;
+#pragma unroll
+            for (int q = 0; q < CW; ++q) s += part[q][j];
+            blk[pass][j] = s;
+        }
+        cl.sync();
+        // four groups of threads take four blocks each, 64 columns at a time
+        for (int j0 = 0; j0 < cols; j0 += 64) {
+            const int g = threadIdx.x >> 6, j = j0 + (threadIdx.x & 63);
+            double s = 0.0;
+            if (j < cols)
+#pragma unroll
+                for (int b = 0; b < CB / 4; ++b) s += *cl.map_shared_rank(&blk[pass][j], g * (CB / 4) + b);
+            fin[g][threadIdx.x & 63] = s;
+            __syncthreads();
+            if (threadIdx.x < 64 && j < cols) {
+                s = (fin[0][threadIdx.x] + fin[1][threadIdx.x]) + (fin[2][threadIdx.x] + fin[3][threadIdx.x]);
+                if (j < k) {
+                    const double sj = sc[SC_SCALE + j], h = s * sj;
+                    c[j] = -h * sj;
+                    if (blockIdx.x == 0) {
+                        if (pass == 0) sc[SC_H1 + j] = h;
+                        host[j] = pass == 0 ? h : sc[SC_H1 + j] + h;
+                    }
+                } else {
+                    bn[0] = s;   // |w|^2 before
+                }
+            }
+            __syncthreads();
+        }
+        double nn = 0.0;
+#pragma unroll
+        for (int p = 0; p < CP; ++p) {
+            if (at[p] < 0) break;
+            double2 s = x[p];
+            for (int j0 = 0; j0 < k; j0 += 8) {
+                double2 v[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t)
+                    if (j0 + t < k) v[t] = load2(V + (size_t)(j0 + t) * ld, at[p], n);
+#pragma unroll
+                for (int t = 0; t < 8; ++t)
+                    if (j0 + t < k) {
+                        s.x = fma(c[j0 + t], v[t].x, s.x);
+                        s.y = fma(c[j0 + t], v[t].y, s.y);
+                    }
+            }
+            x[p] = s;
+            nn = fma(s.y, s.y, fma(s.x, s.x, nn));
+        }
+        __syncwarp();
+        if (busy) nn = warp_sum(nn);
+        if (lane == 0) nrm[pass][warp] = nn;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+#pragma unroll
+            for (int q = 0; q < CW; ++q) s += nrm[pass][q];
+            blk[pass][256] = s;
+        }
+        cl.sync();
+        if (warp == 0) {
+            double s = lane < CB ? *cl.map_shared_rank(&blk[pass][256], lane) : 0.0;
+#pragma unroll
+            for (int o = CB / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) bn[1] = s;
+        }
+        __syncthreads();
+        tot = bn[1];
+        if (!(tot < thr * bn[0])) break;   // the same numbers in every block: all leave together
+    }
+#pragma unroll
+    for (int p = 0; p < CP; ++p) {
+        if (at[p] < 0) break;
+        if (at[p] + 1 < n) *reinterpret_cast<double2*>(w + at[p]) = x[p];
+        else w[at[p]] = x[p].x;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        host[SC_NA] = tot;
+        sc[SC_SCALE + k] = tot > 0.0 ? 1.0 / sqrt(tot) : 0.0;
+    }
+    __threadfence_system();
+    cl.sync();   // no block leaves while its sums may still be read
+}
+cudaError_t launch_cluster(double* V, int64_t ld, int k, const Source& src, int64_t n, double* sc, double thr, double* host,
+                           cudaStream_t st) {
+    // a cluster of 16 is more than every device has to offer: the kernel says that it wants one
+    static const cudaError_t allowed = cudaFuncSetAttribute(cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (allowed != cudaSuccess) return allowed;
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeClusterDimension;
+    a.val.clusterDim = {CB, 1, 1};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(CB);
+    cfg.blockDim = dim3(CT);
+    cfg.stream = st;
+    cfg.attrs = &a;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, cluster_kernel, V, ld, k, src, n, sc, thr, host);
+}
+
 // u = sum_{j<k} y_j v_j
 __global__ void combine_kernel(const double* __restrict__ V, int64_t ld, int k, const double* __restrict__ y,
                                const double* __restrict__ scale, double* __restrict__ u, int64_t n) {
@@ -242,6 +418,13 @@ void launch_dots(int kk, int nb, int th, const double* V, int64_t ld, const Sour
 
 int orthogonalise(double* V, int64_t ld, int k, const Source& src, int64_t n, double* sc, double thr, double* host, double* partials,
                   unsigned int* counter, cudaStream_t st) {
+    // one cluster: 16 of the SMs, so only while their FP64 pipes are quicker than four launches.
+    // Arnoldi step at 20 and 40 columns: n = 5,445: 25, 34 us against 41, 56; 15,765: 30, 44 against
+    // 46, 68; 29,478: 46, 72 against 57, 87 (both sides grow with n k from there)
+    if (n <= CLUSTER_N) {
+        launch_cluster(V, ld, k, src, n, sc, thr, host, st);   // the caller asks for the launch error
+        return 1;
+    }
     // small vectors take two-warp blocks: the reductions are FP64 work per block, and the FP64 pipe
     // is per SM
     const int64_t sms = chns_num_sms();

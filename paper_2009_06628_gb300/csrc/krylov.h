@@ -55,7 +55,8 @@ struct Source {
 // Gram-Schmidt of w (slot k of V, or formed there from src) against slots 0..k-1: coefficients,
 // norms and s_k in sc; host (pinned) gets the coefficients of both passes together in [0, k) and
 // |w|^2 in [SC_NA].  thr: re-orthogonalise when |w|^2 falls below thr times its old value (infinity:
-// always).  Four launches, and two more per 32 columns beyond 32; returns their number.
+// always).  One launch for short vectors; else four, and two more per 32 columns beyond 32; returns
+// their number.
 // partials: 33 doubles for each of 16 blocks per SM; counter: zero.
 int orthogonalise(double* V, int64_t ld, int k, const Source& src, int64_t n, double* sc, double thr, double* host, double* partials,
                   unsigned int* counter, cudaStream_t st);

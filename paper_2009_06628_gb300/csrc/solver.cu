@@ -570,20 +570,18 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
         auto apply_op = [&](int j, int es) -> chns_status {
             const double *Vj = ws->V + (size_t)j * ws->ld, *sj = ws->sc + SC_SCALE + j;
             cudaEvent_t* E = ws->ev + 8 * es;
-            CHNS_CUDA(cudaEventRecord(E[4], c.s));
+            if (j == 0) CHNS_CUDA(cudaEventRecord(E[4], c.s));   // later ones start where the Gram-Schmidt pass ended
             if (mixed) {
                 launch_pc_first<false>(m, pcmask, ws->Pinv32, Vj, sj, ws->Sd, ws->z32, c.s);
                 if (schur && (st = precond_apply(m, spec, ws->z32, pmn, c.s)) != CHNS_OK) return st;
                 if (pin == 2 && !schur) pmean(ws->z32);
                 CHNS_CUDA(cudaEventRecord(E[5], c.s));
-                CHNS_CUDA(cudaEventRecord(E[0], c.s));
                 CHNS_CUDA(launch_jvp32(m, pc, ws->Uo32, ws->Us32, ws->z32, ws->y32, pin, c.s));
             } else {
                 launch_pc_first<false>(m, pcmask, ws->Pinv64, Vj, sj, ws->Sd, ws->z64, c.s);
                 if (schur && (st = precond_apply(m, spec, ws->z64, pmn, c.s)) != CHNS_OK) return st;
                 if (pin == 2 && !schur) pmean(ws->z64);
                 CHNS_CUDA(cudaEventRecord(E[5], c.s));
-                CHNS_CUDA(cudaEventRecord(E[0], c.s));
                 CHNS_CUDA(launch_jvp64(m, pc, U_old, U, ws->z64, ws->t64, pin, c.s));
             }
             CHNS_CUDA(cudaEventRecord(E[1], c.s));
@@ -604,25 +602,23 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
                 const int es = j & 1;
                 // classical Gram-Schmidt with selective re-orthogonalisation (decided on the
                 // device) and the next Arnoldi vector, all queued without a host round trip
-                CHNS_CUDA(cudaEventRecord(ws->ev[6], c.s));
+                cudaEvent_t* E = ws->ev + 8 * es;
                 chns_count_launches(orth_enqueue(c.s, j));
                 CHNS_CUDA(cudaGetLastError());
-                CHNS_CUDA(cudaEventRecord(ws->ev[7], c.s));
-                CHNS_CUDA(cudaEventRecord(ws->ev[10], c.s));
+                CHNS_CUDA(cudaEventRecord(E[7], c.s));
                 // queue the next vector's operator application before reading the scalars, so
                 // the GPU works on it while the host updates the Hessenberg column; if this
                 // iteration turns out to be the last one, that result is simply not used
                 if (j + 1 < mres && kry + 1 < o->max_krylov)
                     if ((st = apply_op(j + 1, es ^ 1)) != CHNS_OK) return st;
-                CHNS_CUDA(cudaEventSynchronize(ws->ev[10]));
+                CHNS_CUDA(cudaEventSynchronize(E[7]));
                 {
-                    cudaEvent_t* E = ws->ev + 8 * es;
                     float ms = 0.0f;
-                    CHNS_CUDA(cudaEventElapsedTime(&ms, E[0], E[1]));
+                    CHNS_CUDA(cudaEventElapsedTime(&ms, E[5], E[1]));
                     S.jvp_ms += ms;
-                    CHNS_CUDA(cudaEventElapsedTime(&ms, E[4], E[5]));
+                    CHNS_CUDA(cudaEventElapsedTime(&ms, j == 0 ? E[4] : ws->ev[8 * (es ^ 1) + 7], E[5]));
                     S.apply_ms += ms;
-                    CHNS_CUDA(cudaEventElapsedTime(&ms, ws->ev[6], ws->ev[7]));
+                    CHNS_CUDA(cudaEventElapsedTime(&ms, E[1], E[7]));
                     S.orth_ms += ms;
                     if (pc_pending) {
                         CHNS_CUDA(cudaEventElapsedTime(&ms, ws->ev[2], ws->ev[3]));

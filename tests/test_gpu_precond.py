@@ -121,3 +121,25 @@ def test_arnoldi_over_column_counts(chns, dim, level, restart, its):
     true = float((gn - g).norm())
     assert 0.0 < st.res_final < float(g.norm()) and abs(true - st.res_final) <= 0.01 * st.res_final, (true, st.as_dict())
     assert float((go + gold).norm()) <= 1e-12 * float(gold.norm()) and abs(float(gc + gcn)) <= 1e-11 * abs(float(gcn))
+
+
+@pytest.mark.parametrize("dim,lmin,level,its", [(2, 4, 4, 40), (2, 5, 5, 9), (2, 4, 7, 40), (3, 3, 3, 70), (3, 2, 4, 33),
+                                                (2, 5, 7, 40), (3, 4, 4, 40)])
+def test_arnoldi_over_vector_lengths(chns, dim, lmin, level, its):
+    """Vectors of 1,445 to 29,478 values, odd and even: one cluster with one and two entry pairs per
+    thread, and past its range two-warp blocks.  The claim and its bound are those of the test over
+    column counts: the reported residual is the true one to 1 %."""
+    import ctypes
+    leaves = synth.uniform_leaves(dim, level) if lmin == level else \
+        synth.sphere_band_leaves(dim, lmin, level, [[0.5] * dim], [0.25], 0.04)
+    gm, prm, U0 = problem(chns, dim, leaves, level, "drop3d" if dim == 3 else "drop2d", Cn=0.08, rho_ratio=3.0, eta_ratio=2.0,
+                          Fr=1.0, dt=1e-4, pin_pressure=1)
+    g = torch.tensor(synth.random_vectors(U0.numel(), 1, 5)[0], device="cuda").reshape(U0.shape)
+    o = chns.SolverOpts.make(krylov_rtol=1e-6, restart=256, max_krylov=its, pc_type=0)
+    lam, go, st = torch.empty_like(g), torch.empty_like(g), chns.Stats()
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr())
+    code = chns.load().chns_step_adjoint(gm.handle, ctypes.byref(prm), ctypes.byref(o), ptr(U0), ptr(U0), ptr(g), ptr(lam),
+                                         ptr(go), None, ctypes.byref(st), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert chns.STATUS[code] in ("CHNS_OK", "CHNS_ENOCONV")
+    true = float((chns.vjp(gm, prm, U0, U0, lam)[0] - g).norm())
+    assert 0.0 < st.res_final < float(g.norm()) and abs(true - st.res_final) <= 0.01 * st.res_final, (true, st.as_dict())
