@@ -130,9 +130,6 @@ void transfer_free(TransferDev* T);
 // FP64, overwriting out
 cudaError_t transfer_apply_f64(const TransferDev& T, bool transpose, int nf, const double* in, double* out,
                                cudaStream_t s);
-// scalar FP32 fields: out (+)= P in or P^T in
-cudaError_t transfer_apply_f32(const TransferDev& T, bool transpose, bool add, const float* in, float* out,
-                               cudaStream_t s);
 
 // Geometric multigrid hierarchy of the pressure Schur Laplacian (multigrid.cu builds it,
 // precond.cu assembles its levels and applies V-cycles).  Level 0 is the mesh itself; level l + 1 caps

@@ -368,8 +368,8 @@ __global__ void __launch_bounds__(CT, 1) cluster_kernel(double* V, int64_t ld, i
 }
 cudaError_t launch_cluster(double* V, int64_t ld, int k, const Source& src, int64_t n, double* sc, double thr, double* host,
                            cudaStream_t st) {
-    // a cluster of 16 is more than every device has to offer: the kernel says that it wants one
-    static const cudaError_t allowed = cudaFuncSetAttribute(cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    // more than 8 blocks are a cluster only where the kernel allows it, on this device
+    const cudaError_t allowed = cudaFuncSetAttribute(cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (allowed != cudaSuccess) return allowed;
     cudaLaunchAttribute a;
     a.id = cudaLaunchAttributeClusterDimension;
@@ -422,8 +422,8 @@ int orthogonalise(double* V, int64_t ld, int k, const Source& src, int64_t n, do
     // Arnoldi step at 20 and 40 columns: n = 5,445: 25, 34 us against 41, 56; 15,765: 30, 44 against
     // 46, 68; 29,478: 46, 72 against 57, 87 (both sides grow with n k from there)
     if (n <= CLUSTER_N) {
-        launch_cluster(V, ld, k, src, n, sc, thr, host, st);   // the caller asks for the launch error
-        return 1;
+        if (launch_cluster(V, ld, k, src, n, sc, thr, host, st) == cudaSuccess) return 1;
+        (void)cudaGetLastError();   // no room for the cluster (a partitioned device): the general kernels
     }
     // small vectors take two-warp blocks: the reductions are FP64 work per block, and the FP64 pipe
     // is per SM

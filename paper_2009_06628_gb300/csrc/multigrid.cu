@@ -35,19 +35,15 @@ cudaError_t upload(T** dst, const std::vector<T>& src) {
     return e;
 }
 
-// y[row] (+)= sum_j w_j x[col_j] for every field f < nf of node-major vectors
-template <class T, class W, bool ADD>
+// y[row] = sum_j w_j x[col_j] for every field f < nf of node-major vectors
 __global__ void csr_apply_kernel(int64_t rows, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                                 const W* __restrict__ w, int nf, const T* __restrict__ x, T* __restrict__ y) {
+                                 const double* __restrict__ w, int nf, const double* __restrict__ x, double* __restrict__ y) {
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j0 = rp[r], j1 = rp[r + 1];
         for (int f = 0; f < nf; ++f) {
-            T acc = T(0);
-            for (int64_t j = j0; j < j1; ++j) acc += (T)w[j] * x[(size_t)col[j] * nf + f];
-            if (ADD)
-                y[(size_t)r * nf + f] += acc;
-            else
-                y[(size_t)r * nf + f] = acc;
+            double acc = 0.0;
+            for (int64_t j = j0; j < j1; ++j) acc += w[j] * x[(size_t)col[j] * nf + f];
+            y[(size_t)r * nf + f] = acc;
         }
     }
 }
@@ -194,23 +190,9 @@ cudaError_t transfer_apply_f64(const TransferDev& T, bool transpose, int nf, con
                                cudaStream_t s) {
     const int64_t rows = transpose ? T.n_src : T.n_dst;
     if (transpose)
-        csr_apply_kernel<double, double, false><<<grid_rows(rows), 256, 0, s>>>(rows, T.rpT, T.colT, T.wT, nf, in, out);
+        csr_apply_kernel<<<grid_rows(rows), 256, 0, s>>>(rows, T.rpT, T.colT, T.wT, nf, in, out);
     else
-        csr_apply_kernel<double, double, false><<<grid_rows(rows), 256, 0, s>>>(rows, T.rp, T.col, T.w, nf, in, out);
-    chns_count_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t transfer_apply_f32(const TransferDev& T, bool transpose, bool add, const float* in, float* out,
-                               cudaStream_t s) {
-    const int64_t rows = transpose ? T.n_src : T.n_dst;
-    const int64_t* rp = transpose ? T.rpT : T.rp;
-    const int32_t* col = transpose ? T.colT : T.col;
-    const float* w = transpose ? T.wTf : T.wf;
-    if (add)
-        csr_apply_kernel<float, float, true><<<grid_rows(rows), 256, 0, s>>>(rows, rp, col, w, 1, in, out);
-    else
-        csr_apply_kernel<float, float, false><<<grid_rows(rows), 256, 0, s>>>(rows, rp, col, w, 1, in, out);
+        csr_apply_kernel<<<grid_rows(rows), 256, 0, s>>>(rows, T.rp, T.col, T.w, nf, in, out);
     chns_count_launches(1);
     return cudaGetLastError();
 }

@@ -386,6 +386,93 @@ __device__ __forceinline__ int64_t my_row(int64_t N, bool& store) {
     return r < N ? r : N - 1;
 }
 
+// Up to SPLIT_ROWS rows (four lanes each) the launched kernels are links of a chain: each may start
+// while its predecessor runs (programmatic dependent launch), loads what no link changes (matrix,
+// diagonal, coefficients), and waits there.  Every thread waits before it touches a vector, so a link
+// that is done implies that all earlier ones are.  Vectors are then read with plain loads: the
+// read-only path asks that nobody writes them meanwhile.  V-cycle and Cahn-Hilliard block on 45,000
+// rows: 163 -> 139 us.  Larger grids fill the chip, and a successor that waits would take its place.
+template <int LPR> constexpr bool LINK = LPR != 1;
+template <bool ON> __device__ __forceinline__ void chain_next() {
+    if (ON) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <bool ON> __device__ __forceinline__ void chain_wait() {
+    if (ON) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <bool ON> __device__ __forceinline__ float vec(const float* x) { return ON ? *x : __ldg(x); }
+template <bool ON, class... P, class... A>
+void chain(void (*kernel)(P...), int grid, int threads, cudaStream_t st, A... args) {
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cfg.attrs = &a;
+    cfg.numAttrs = ON ? 1 : 0;
+    (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);   // errors: cudaGetLastError at the chain's end
+}
+// A row of this lane group, its first PRE entries per lane already loaded
+template <int LPR>
+struct Row {
+    static constexpr int PRE = 8;
+    const float* v;
+    const int32_t* c;
+    int w, sub;
+    float pv[PRE];
+    int pc[PRE];
+    __device__ __forceinline__ Row(const Sell& S, const float* __restrict__ val, int64_t r) {
+        const int64_t o0 = __ldg(S.off + (r >> 5));
+        w = (int)((__ldg(S.off + (r >> 5) + 1) - o0) >> 5);
+        sub = threadIdx.x % LPR;
+        v = val + o0 + (r & 31);
+        c = S.col + o0 + (r & 31);
+#pragma unroll
+        for (int i = 0; i < PRE; ++i) {
+            const int j = sub + i * LPR;
+            pv[i] = j < w ? __ldg(v + (int64_t)j * 32) : 0.0f;
+            pc[i] = j < w ? __ldg(c + (int64_t)j * 32) : (int)r;
+        }
+    }
+    // a column scaling that no link changes
+    __device__ __forceinline__ void scale(const float* __restrict__ d) {
+#pragma unroll
+        for (int i = 0; i < PRE; ++i) pv[i] *= __ldg(d + pc[i]);
+    }
+    // sum_j a_j x_j: x(column) for the loaded entries; scaled(column) brings the scaling along
+    template <class X, class Scaled>
+    __device__ __forceinline__ float dot(X x, Scaled scaled) const {
+        float s = 0.0f;
+#pragma unroll
+        for (int i = 0; i < PRE; ++i) s = fmaf(pv[i], x(pc[i]), s);
+#pragma unroll 8
+        for (int j = sub + PRE * LPR; j < w; j += LPR) s = fmaf(__ldg(v + (int64_t)j * 32), scaled(__ldg(c + (int64_t)j * 32)), s);
+#pragma unroll
+        for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, LPR);
+        return s;
+    }
+    __device__ __forceinline__ float dot(const float* x) const {
+        const auto at = [&](int q) { return x[q]; };
+        return dot(at, at);
+    }
+};
+// A lane per row: nothing is loaded ahead.  The kernels are to stay at 32 registers, so that the 1,073
+// blocks of 64^3 are resident at once (40 registers: 7.2 -> 9.6 us per step).
+template <>
+struct Row<1> {
+    const Sell& S;
+    const float* val;
+    int64_t r;
+    __device__ __forceinline__ Row(const Sell& S, const float* val, int64_t r) : S(S), val(val), r(r) {}
+    __device__ __forceinline__ void scale(const float*) {}
+    template <class X, class Scaled>
+    __device__ __forceinline__ float dot(X, Scaled scaled) const { return row_dot<1>(S, val, r, scaled); }
+    __device__ __forceinline__ float dot(const float* x) const {
+        return row_dot<1>(S, val, r, [&](int q) { return __ldg(x + q); });
+    }
+};
+
 // Adds m_n z_n of a block's threads to its partial; the block that finishes last sums the
 // partials in a fixed order.  All threads of the block call it.
 __device__ __forceinline__ void mean_add(const PrecondMean& M, double v) {
@@ -428,21 +515,35 @@ __device__ __forceinline__ void mean_add(const PrecondMean& M, double v) {
 // and d = dinv b / theta is formed where it is gathered, x = 0.  LAST: the result base + x + d + d'
 // goes to z (strided field f; z may be base, base may be null) and r, d' are not kept.
 template <int LPR, bool FIRST, bool LAST, class TO>
-__global__ void __launch_bounds__(256) cheb_step_kernel(Sell S, const float* __restrict__ val,
+__global__ void __launch_bounds__(256, LPR == 1 ? 8 : 1) cheb_step_kernel(Sell S, const float* __restrict__ val,
                                                         const float* __restrict__ dinv,
-                                                        const ChebCoef* __restrict__ cf, int k,
-                                                        const float* __restrict__ b, const float* __restrict__ d,
-                                                        float* __restrict__ dn, float* __restrict__ r,
-                                                        float* __restrict__ x, const float* base, TO* z, int NF, int f,
-                                                        PrecondMean mean) {
+                                                        const ChebCoef* __restrict__ cf, int k, const float* b,
+                                                        const float* d, float* dn, float* r, float* x, const float* base,
+                                                        TO* z, int NF, int f, PrecondMean mean) {
+    chain_next<LINK<LPR>>();
     bool store;
     const int64_t n = my_row<LPR>(S.N, store);
-    const float di = dinv[n], it = FIRST ? cf->inv_theta : 0.0f;
-    const float rr = FIRST ? b[n] : r[n], dd = FIRST ? it * di * rr : d[n], xx = FIRST ? 0.0f : x[n];
-    float y;
-    if (FIRST) y = row_dot<LPR>(S, val, n, [&](int q) { return it * __ldg(dinv + q) * __ldg(b + q); });
-    else y = row_dot<LPR>(S, val, n, [&](int q) { return __ldg(d + q); });
-    const float rn = rr - y, dv = cf->c1[k] * dd + cf->c2[k] * di * rn;
+    float di, it, rr, dd, xx, y, c1, c2;
+    const auto own = [&] {
+        rr = FIRST ? b[n] : r[n];
+        dd = FIRST ? it * di * rr : d[n];
+        xx = FIRST ? 0.0f : x[n];
+    };
+    if constexpr (LINK<LPR>) {
+        Row<LPR> row(S, val, n);
+        di = dinv[n], it = FIRST ? cf->inv_theta : 0.0f, c1 = cf->c1[k], c2 = cf->c2[k];
+        if (FIRST) row.scale(dinv);
+        chain_wait<true>();
+        own();
+        y = FIRST ? it * row.dot([&](int q) { return b[q]; }, [&](int q) { return __ldg(dinv + q) * b[q]; }) : row.dot(d);
+    } else {
+        di = dinv[n], it = FIRST ? cf->inv_theta : 0.0f;
+        own();
+        if (FIRST) y = row_dot<1>(S, val, n, [&](int q) { return it * __ldg(dinv + q) * __ldg(b + q); });
+        else y = row_dot<1>(S, val, n, [&](int q) { return __ldg(d + q); });
+        c1 = cf->c1[k], c2 = cf->c2[k];
+    }
+    const float rn = rr - y, dv = c1 * dd + c2 * di * rn;
     if (LAST) {
         const float v = base ? base[n] + ((xx + dd) + dv) : (xx + dd) + dv;
         if (store) z[(size_t)n * NF + f] = (TO)v;
@@ -455,34 +556,64 @@ __global__ void __launch_bounds__(256) cheb_step_kernel(Sell S, const float* __r
 }
 // t = b - A x (t may be b)
 template <int LPR>
-__global__ void __launch_bounds__(256) residual_kernel(Sell S, const float* __restrict__ val, const float* b,
-                                                       const float* __restrict__ x, float* t) {
+__global__ void __launch_bounds__(256, LPR == 1 ? 8 : 1) residual_kernel(Sell S, const float* __restrict__ val, const float* b, const float* x,
+                                                       float* t) {
+    chain_next<LINK<LPR>>();
     bool store;
     const int64_t n = my_row<LPR>(S.N, store);
-    const float y = row_dot<LPR>(S, val, n, [&](int q) { return __ldg(x + q); });
+    const Row<LPR> row(S, val, n);
+    chain_wait<LINK<LPR>>();
+    const float y = row.dot(x);
     if (store) t[n] = b[n] - y;
+}
+// y (+)= A x for the transfers between levels (compressed rows, 8 lanes each), a link of the chain too
+template <bool ADD>
+__global__ void __launch_bounds__(256) transfer_kernel(int64_t N, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
+                                                       const float* __restrict__ w, const float* x, float* y) {
+    constexpr int L = 8, PRE = 4;
+    chain_next<true>();
+    bool store;
+    const int64_t n = my_row<L>(N, store), j0 = __ldg(rp + n) + threadIdx.x % L, j1 = __ldg(rp + n + 1);
+    float v[PRE], s = 0.0f;
+    int c[PRE];
+#pragma unroll
+    for (int i = 0; i < PRE; ++i) {
+        const bool has = j0 + i * L < j1;
+        v[i] = has ? __ldg(w + j0 + i * L) : 0.0f;
+        c[i] = has ? __ldg(col + j0 + i * L) : -1;
+    }
+    chain_wait<true>();
+#pragma unroll
+    for (int i = 0; i < PRE; ++i) s = fmaf(v[i], c[i] < 0 ? 0.0f : x[c[i]], s);
+    for (int64_t j = j0 + PRE * L; j < j1; j += L) s = fmaf(__ldg(w + j), x[__ldg(col + j)], s);
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, L);
+    if (store) y[n] = ADD ? y[n] + s : s;
 }
 // r = base + c A (x .* m): the right-hand side of a Chebyshev solve (base, m may be null)
 template <int LPR>
-__global__ void __launch_bounds__(256) rhs_kernel(Sell S, const float* __restrict__ val, const float* __restrict__ x,
-                                                  const float* __restrict__ m, const float* __restrict__ base, float c,
-                                                  float* __restrict__ r) {
+__global__ void __launch_bounds__(256, LPR == 1 ? 8 : 1) rhs_kernel(Sell S, const float* __restrict__ val, const float* x,
+                                                  const float* __restrict__ m, const float* base, float c, float* r) {
+    chain_next<LINK<LPR>>();
     bool store;
     const int64_t n = my_row<LPR>(S.N, store);
-    float y;
-    if (m) y = row_dot<LPR>(S, val, n, [&](int q) { return __ldg(m + q) * __ldg(x + q); });
-    else y = row_dot<LPR>(S, val, n, [&](int q) { return __ldg(x + q); });
+    Row<LPR> row(S, val, n);
+    if (m) row.scale(m);
+    chain_wait<LINK<LPR>>();
+    const float y = m ? row.dot([&](int q) { return vec<LINK<LPR>>(x + q); }, [&](int q) { return __ldg(m + q) * vec<LINK<LPR>>(x + q); }) : row.dot(x);
     if (store) r[n] = base ? base[n] + c * y : c * y;
 }
 // Cahn-Hilliard block, last pass: z_phi = x, z_mu = psi2 x + (Cn^2 K x - 2 r_mu) / m_l (lumped mass)
 template <int LPR, class TO>
-__global__ void __launch_bounds__(256) ch_store_kernel(Sell S, const float* __restrict__ vk, int NF, int fphi,
-                                                       const float* __restrict__ x, const float* __restrict__ rm,
-                                                       const float* __restrict__ psi2, const float* __restrict__ iml,
-                                                       float cn2, TO* __restrict__ z) {
+__global__ void __launch_bounds__(256, LPR == 1 ? 8 : 1) ch_store_kernel(Sell S, const float* __restrict__ vk, int NF, int fphi, const float* x,
+                                                       const float* rm, const float* psi2, const float* __restrict__ iml,
+                                                       float cn2, TO* z) {
+    chain_next<LINK<LPR>>();
     bool store;
     const int64_t n = my_row<LPR>(S.N, store);
-    const float kx = row_dot<LPR>(S, vk, n, [&](int q) { return __ldg(x + q); });
+    const Row<LPR> row(S, vk, n);
+    chain_wait<LINK<LPR>>();
+    const float kx = row.dot(x);
     if (!store) return;
     const float xv = x[n], il = iml[n];
     z[(size_t)n * NF + fphi] = (TO)xv;
@@ -656,6 +787,8 @@ template <class TO>
 __global__ void __launch_bounds__(TAIL_THREADS) tail_kernel(const Tail* __restrict__ tp, TO* __restrict__ z, int NF, int f,
                                                             PrecondMean mean) {
     __shared__ float sd[2][TAIL_ROWS];
+    chain_next<true>();
+    chain_wait<true>();
     const Tail& T = *tp;
     const int64_t t0 = threadIdx.x, nt = TAIL_THREADS;
     for (int l = 0; l + 1 < T.n; ++l) {
@@ -932,7 +1065,7 @@ void split(int64_t N, F f) {
 void launch_residual_rows(const Level& L, float* t, cudaStream_t st) {   // t = b - A x
     split(L.dm.N, [&](auto lpr) {
         constexpr int LPR = decltype(lpr)::value;
-        residual_kernel<LPR><<<blocks_for(L.dm.N * LPR), 256, 0, st>>>(L.S, L.val, L.b, L.x, t);
+        chain<LINK<LPR>>(residual_kernel<LPR>, blocks_for(L.dm.N * LPR), 256, st, L.S, L.val, L.b, L.x, t);
     });
 }
 
@@ -946,8 +1079,8 @@ int cheb(const Sell& S, const float* val, const float* dinv, const ChebCoef* cf,
         for (int k = 0; k + 1 < deg; ++k) {
             const bool last = k + 2 == deg;
             auto run = [&](auto first, auto fin) {
-                cheb_step_kernel<LPR, decltype(first)::value, decltype(fin)::value, TO><<<g, 256, 0, st>>>(
-                    S, val, dinv, cf, k, b, d0, d1, r, x, base, z, NF, f, mean);
+                chain<LINK<LPR>>(cheb_step_kernel<LPR, decltype(first)::value, decltype(fin)::value, TO>, g, 256, st, S, val, dinv, cf, k, b, d0,
+                      d1, r, x, base, z, NF, f, mean);
             };
             if (k == 0 && last) run(std::true_type(), std::true_type());
             else if (k == 0) run(std::true_type(), std::false_type());
@@ -975,17 +1108,17 @@ cudaError_t vcycle(chns_mesh* m, const PrecondSpec& spec, TO* z, int NF, int f, 
         Level& L = p->lv[(size_t)l];
         *nk += smooth<float>(L, p->cf + l, spec.degree, nullptr, L.x, 1, 0, PrecondMean(), st);
         launch_residual_rows(L, L.t, st);
-        const cudaError_t e = transfer_apply_f32(m->mg->lv[(size_t)l + 1].P, true, false, L.t, p->lv[(size_t)l + 1].b, st);
-        if (e != cudaSuccess) return e;
+        const TransferDev& P = m->mg->lv[(size_t)l + 1].P;
+        chain<true>(transfer_kernel<false>, blocks_for(P.n_src * 8), 256, st, P.n_src, P.rpT, P.colT, P.wTf, L.t, p->lv[(size_t)l + 1].b);
         *nk += 2;
     }
     const bool all = from == 0;   // every level runs in the one block
-    tail_kernel<TO><<<1, TAIL_THREADS, 0, st>>>(p->tail, all ? z : nullptr, NF, f, all ? mean : PrecondMean());
+    chain<true>(tail_kernel<TO>, 1, TAIL_THREADS, st, p->tail, all ? z : nullptr, NF, f, all ? mean : PrecondMean());
     ++*nk;
     for (int l = from - 1; l >= 0; --l) {
         Level& L = p->lv[(size_t)l];
-        const cudaError_t e = transfer_apply_f32(m->mg->lv[(size_t)l + 1].P, false, true, p->lv[(size_t)l + 1].x, L.x, st);
-        if (e != cudaSuccess) return e;
+        const TransferDev& P = m->mg->lv[(size_t)l + 1].P;
+        chain<true>(transfer_kernel<true>, blocks_for(P.n_dst * 8), 256, st, P.n_dst, P.rp, P.col, P.wf, p->lv[(size_t)l + 1].x, L.x);
         launch_residual_rows(L, L.b, st);
         *nk += 2;
         *nk += l == 0 ? smooth<TO>(L, p->cf, spec.degree, L.x, z, NF, f, mean, st)
@@ -999,7 +1132,7 @@ cudaError_t polynomial(chns_mesh* m, const PrecondSpec& spec, TO* z, int NF, int
     PrecondWS* p = m->pre;
     Level& L = p->lv[0];
     if (p->tail_from == 0) {
-        tail_kernel<TO><<<1, TAIL_THREADS, 0, st>>>(p->tail, z, NF, f, mean);
+        chain<true>(tail_kernel<TO>, 1, TAIL_THREADS, st, p->tail, z, NF, f, mean);
         ++*nk;
         return cudaGetLastError();
     }
@@ -1015,7 +1148,7 @@ cudaError_t cahn_hilliard(chns_mesh* m, const PrecondSpec& spec, TO* z, int NF, 
     auto rhs = [&](const float* val, const float* x, const float* mul, const float* base, float a, float* r) {
         split(N, [&](auto lpr) {
             constexpr int LPR = decltype(lpr)::value;
-            rhs_kernel<LPR><<<blocks_for(N * LPR), 256, 0, st>>>(p->SC, val, x, mul, base, a, r);
+            chain<LINK<LPR>>(rhs_kernel<LPR>, blocks_for(N * LPR), 256, st, p->SC, val, x, mul, base, a, r);
         });
     };
     auto solve = [&](const float* b, float* x) {   // (M + eps K)^{-1} b
@@ -1027,7 +1160,7 @@ cudaError_t cahn_hilliard(chns_mesh* m, const PrecondSpec& spec, TO* z, int NF, 
     *nk += 2 + solve(p->cb, p->ca);
     split(N, [&](auto lpr) {
         constexpr int LPR = decltype(lpr)::value;
-        ch_store_kernel<LPR, TO><<<blocks_for(N * LPR), 256, 0, st>>>(p->SC, p->vk, NF, f, p->ca, p->rm, p->psi2, p->iml, spec.cn2, z);
+        chain<LINK<LPR>>(ch_store_kernel<LPR, TO>, blocks_for(N * LPR), 256, st, p->SC, p->vk, NF, f, p->ca, p->rm, p->psi2, p->iml, spec.cn2, z);
     });
     return cudaGetLastError();
 }
