@@ -202,6 +202,7 @@ elem_rj_kernel(DevMesh m, const __grid_constant__ Q1Params<S> prm, const typenam
         S r[NF];
 #pragma unroll
         for (int f = 0; f < NF; ++f) r[f] = mul2(L.vol, q1_vgradT<D, false>(prm.f, prm.fr, F0[f], F1[f], (const S*)nullptr));
+        chain_wait<true>();
 #pragma unroll
         for (int h = 0; h < NP; ++h) {
             T rh[NF];
@@ -332,6 +333,7 @@ elem_vjp_kernel(DevMesh m, const __grid_constant__ Q1Params<double> prm, double 
             ro[k] = fma(-L.vol, b, a);
         }
     }
+    chain_wait<true>();
     {
         const Parents P = parents_of(m, ent);
         const double wt = parent_weight<double>(P.n);
@@ -404,10 +406,10 @@ cudaError_t launch_rj(const chns_mesh* mm, const PhysConst& pc, const typename S
     } else {
         const int th = ek_threads(m.E * LPE);
         if (mm->scatter == SCAT_WARPAGG)
-            elem_rj_kernel<D, S, MODE, SCAT_WARPAGG><<<grid(m.E, th), th, 0, s>>>(
+            chain<true>(elem_rj_kernel<D, S, MODE, SCAT_WARPAGG>, grid(m.E, th), th, s,
                 m, prm, Uo, Un, x, out, mm->d_flags, nullptr, m.E, 0, pin);
         else
-            elem_rj_kernel<D, S, MODE, SCAT_ATOMIC><<<grid(m.E, th), th, 0, s>>>(
+            chain<true>(elem_rj_kernel<D, S, MODE, SCAT_ATOMIC>, grid(m.E, th), th, s,
                 m, prm, Uo, Un, x, out, mm->d_flags, nullptr, m.E, pair_rows, pin);
         chns_count_launches(1);
     }
@@ -453,7 +455,7 @@ cudaError_t launch_vjp(const chns_mesh* mm, const PhysConst& pc, const double* U
             }
         } else {
             const int th = ek_threads(m.E * NC);
-            elem_vjp_kernel<D, SCAT_ATOMIC><<<(unsigned)((m.E * NC + th - 1) / th), th, 0, s>>>(
+            chain<true>(elem_vjp_kernel<D, SCAT_ATOMIC>, (unsigned)((m.E * NC + th - 1) / th), th, s,
                 m, prm, 1.0 / pc.Cn, U_old, U_lin, w, gU_new, gU_old, gCn, pin, nullptr, m.E);
             chns_count_launches(1);
         }

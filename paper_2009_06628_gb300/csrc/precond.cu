@@ -28,6 +28,7 @@
 #include <utility>
 #include <vector>
 
+#include "chain.cuh"
 #include "precond.h"
 
 namespace {
@@ -393,26 +394,7 @@ __device__ __forceinline__ int64_t my_row(int64_t N, bool& store) {
 // read-only path asks that nobody writes them meanwhile.  V-cycle and Cahn-Hilliard block on 45,000
 // rows: 163 -> 139 us.  Larger grids fill the chip, and a successor that waits would take its place.
 template <int LPR> constexpr bool LINK = LPR != 1;
-template <bool ON> __device__ __forceinline__ void chain_next() {
-    if (ON) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-template <bool ON> __device__ __forceinline__ void chain_wait() {
-    if (ON) asm volatile("griddepcontrol.wait;" ::: "memory");
-}
 template <bool ON> __device__ __forceinline__ float vec(const float* x) { return ON ? *x : __ldg(x); }
-template <bool ON, class... P, class... A>
-void chain(void (*kernel)(P...), int grid, int threads, cudaStream_t st, A... args) {
-    cudaLaunchAttribute a;
-    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    a.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.stream = st;
-    cfg.attrs = &a;
-    cfg.numAttrs = ON ? 1 : 0;
-    (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);   // errors: cudaGetLastError at the chain's end
-}
 // A row of this lane group, its first PRE entries per lane already loaded
 template <int LPR>
 struct Row {

@@ -385,6 +385,7 @@ q2_rj_kernel(DevMesh m, const __grid_constant__ Q2Params<S> prm, const typename 
         for (int f = 0; f < NF; ++f)
             r[f] = mul2(L.vol, q2_vgradT<D, false, false, S>(F0[f], F1[f], nullptr, nullptr, splat<S>(0.0), l));
     }
+    chain_wait<true>();
 #pragma unroll
     for (int h = 0; h < H; ++h) {
         if (!P.valid[h]) continue;
@@ -502,6 +503,7 @@ q2_vjp_kernel(DevMesh m, const __grid_constant__ Q2Params<double> prm, double iC
             ro[k] = fma(-L.vol, b, a);
         }
     }
+    chain_wait<true>();
     if (P.valid[0]) {
         if (inside) {
             rn[D + 1] += psb;
@@ -544,7 +546,7 @@ cudaError_t q2_launch_rj(const chns_mesh* mm, const PhysConst& pc, const typenam
     unsigned blocks;
     int th;
     q2_grid<D, Halves<S>::n>(m.E, blocks, th);
-    q2_rj_kernel<D, S, MODE><<<blocks, th, 0, s>>>(m, q2_params<D, S>(pc, ldexp(m.hi - m.lo, -(int)mm->q2_level)), Uo, Un, x,
+    chain<true>(q2_rj_kernel<D, S, MODE>, blocks, th, s, m, q2_params<D, S>(pc, ldexp(m.hi - m.lo, -(int)mm->q2_level)), Uo, Un, x,
                                                    out, mm->d_flags, (uintptr_t)out % 8 == 0);
     chns_count_launches(1);
     return cudaGetLastError();
@@ -558,7 +560,7 @@ cudaError_t q2_launch_vjp_d(const chns_mesh* mm, const PhysConst& pc, const doub
     unsigned blocks;
     int th;
     q2_grid<D, 1>(m.E, blocks, th);
-    q2_vjp_kernel<D><<<blocks, th, 0, s>>>(m, q2_params<D, double>(pc, ldexp(m.hi - m.lo, -(int)mm->q2_level)), 1.0 / pc.Cn, Uo,
+    chain<true>(q2_vjp_kernel<D>, blocks, th, s, m, q2_params<D, double>(pc, ldexp(m.hi - m.lo, -(int)mm->q2_level)), 1.0 / pc.Cn, Uo,
                                            Un, w, gn, go, gCn);
     chns_count_launches(1);
     return cudaGetLastError();

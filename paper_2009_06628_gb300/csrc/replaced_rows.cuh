@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include "chain.cuh"
 #include "chns_internal.h"
 
 namespace {
@@ -21,12 +22,15 @@ __device__ __forceinline__ unsigned replaced_rows(const DevMesh& m, int node, in
 //   J x     : y = x on those rows
 //   J^T w   : g_new = w on those rows, to which the elements add; g_old = -w at the pin
 // One pass in the place of a memset before the elements and a boundary kernel after them: a
-// call is two launches instead of three (five for J^T w), 4 us less of a small call's 23.
+// call is two launches instead of three (five for J^T w), 4 us less of a small call's 23.  The
+// element kernel starts beside it (chain.cuh) and waits for it only where it adds to the output
+// (64^3 FP32 J x: 73 to 69 us; 32^2 FP64: 18.5 to 16.5 us).
 enum { ROWS_RES = 0, ROWS_JVP = 1, ROWS_VJP = 2 };
 template <int D, class T, int MODE>
 __global__ void __launch_bounds__(256) init_rows_kernel(DevMesh m, const T* __restrict__ a, const T* __restrict__ b, T* __restrict__ out,
                                  T* __restrict__ out_old, T* __restrict__ gCn, int pin) {
     constexpr int NF = (D + 3);
+    chain_next<true>();
     // a block covers 256 nodes, entry by entry
     const int64_t node0 = (int64_t)blockIdx.x * 256;
     T* const o = out + node0 * NF;
