@@ -237,8 +237,9 @@ chns_status chns_vjp(const chns_mesh* mesh, const chns_params* params, const dou
  * pressure rows, m_p the nodal masses): nonsingular, with the zero-mean-pressure
  * solution of J dU = -R.  U_old, U_inout: device, N * n_f doubles.  stats: host, may
  * be NULL.  Synchronises the stream (it reads scalars every GMRES iteration).  The
- * first call on a mesh allocates the Krylov workspace; the pressure-Schur apply is
- * captured into CUDA graphs on a private stream of the mesh and replayed on `stream`. */
+ * first call on a mesh allocates the Krylov workspace and, for the spec asked for, the
+ * rows of the preconditioner's matrices; its application is captured into CUDA graphs on
+ * private streams of the mesh and replayed on `stream`. */
 chns_status chns_newton_step(const chns_mesh* mesh, const chns_params* params,
                              const chns_solver_opts* opts, const double* U_old, double* U_inout,
                              chns_stats* stats, void* stream);
@@ -254,8 +255,9 @@ chns_status chns_energy(const chns_mesh* mesh, const chns_params* params, const 
 
 /* Consistent initial chemical potential: overwrite the mu field of U_inout (device)
  * with the solution of M mu = (N, psi'(phi)) + Cn^2 (grad N, grad phi), the potential
- * equation at one time level (Definition 1), by Jacobi-preconditioned CG to a
- * relative residual of 1e-14.  Synchronises the stream. */
+ * equation at one time level (Definition 1), by preconditioned CG to a relative
+ * residual of 1e-14.  The first call on a mesh allocates its workspace (seven node
+ * vectors, kept until chns_mesh_destroy).  Synchronises the stream. */
 chns_status chns_initial_mu(const chns_mesh* mesh, const chns_params* params, double* U_inout,
                             void* stream);
 
@@ -289,7 +291,8 @@ chns_status chns_mu_rhs_vjp(const chns_mesh* mesh, const chns_params* params, co
                             double* g_phi, double* dCn, void* stream);
 
 /* x = M^{-1} rhs with the consistent Q1 mass matrix (CG to 1e-14; M is symmetric, so
- * this is also its adjoint).  rhs, x: device N doubles.  Synchronises the stream. */
+ * this is also its adjoint).  rhs, x: device N doubles, workspace as chns_initial_mu.
+ * Synchronises the stream. */
 chns_status chns_mass_solve(const chns_mesh* mesh, const double* rhs, double* x, void* stream);
 
 /* Integral of phi (as chns_mass) for callers that cannot allocate device memory when
