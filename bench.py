@@ -37,7 +37,8 @@ WORKLOAD = ("3D CHNS drop, uniform octree level 6 (64^3 Q1 hexes, 274,625 nodes 
 METRIC = "CHNS JÂ·x GDOF/s & % HBM roofline; mixed vs FP64 Newton step time at â‰¤1e-9 rel"
 # Per-element counts of the element kernels taken by ncu from one launch on the 64^3 mesh
 # (profiles/element_kernels_64cubed_counts.md): executed floating-point operations (2 x FMA
-# + ADD + MUL thread instructions of the kernel's precision, divided by the element count)
+# + ADD + MUL thread instructions of the kernel's precision, packed FP32 pairs counted twice,
+# divided by the element count)
 # and DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch.  They belong to
 # the kernel sources whose SHA-256 is KERNEL_SRC_SHA; when the sources change, the bench
 # reports them as null (stale) until they are captured again.
@@ -45,12 +46,12 @@ METRIC = "CHNS JÂ·x GDOF/s & % HBM roofline; mixed vs FP64 Newton step time at â
 BENCH_PC_TYPE = 1
 KERNEL_SRC_FILES = tuple("paper_2009_06628_gb300/csrc/" + f for f in ("element_kernels.cu", "point_physics.cuh", "q1_lanes.cuh",
                                                                        "replaced_rows.cuh"))
-KERNEL_SRC_SHA = "de8fd3eb9c4ab80e"
+KERNEL_SRC_SHA = "a9fc2b7a475ce52b"
 KERNEL_COUNTS = {
-    "jvp_fp32": {"flop_per_element": 14769.6, "dram_bytes": 35048192},
-    "jvp_fp64": {"flop_per_element": 15168.0, "dram_bytes": 61910016},
-    "residual_fp64": {"flop_per_element": 9688.0, "dram_bytes": 48285440},
-    "vjp_fp64": {"flop_per_element": 20776.0, "dram_bytes": 77077760},
+    "jvp_fp32": {"flop_per_element": 6886.9, "dram_bytes": 35323904},
+    "jvp_fp64": {"flop_per_element": 7486.9, "dram_bytes": 62303232},
+    "residual_fp64": {"flop_per_element": 4406.9, "dram_bytes": 48532224},
+    "vjp_fp64": {"flop_per_element": 8472.0, "dram_bytes": 77266688},
 }
 
 
