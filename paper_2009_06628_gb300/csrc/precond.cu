@@ -8,9 +8,9 @@
 // arithmetic.  Element-wise, a step was two kernels (8 gathers and 8 atomics per element into a
 // zeroed vector, then the vector update that the atomics have to wait for).  With rows, one
 // kernel gathers, reduces and updates: half the chain, no atomics, a fixed summation order.
-//   64^3 (274,625 rows), degree 16: a whole preconditioner application 313 -> 165 us (of which
-//   about 45 us are the block-Jacobi part); 45,000 rows with hanging points, V-cycle and
-//   Cahn-Hilliard block: 620 -> 195 us; 1,089 rows in 2D, degree 16: 82 -> 56 us.
+//   64^3 (274,625 rows), degree 16: a whole preconditioner application 313 -> 125 us (15 of them the
+//   block-Jacobi part); 45,000 rows with hanging points, V-cycle and Cahn-Hilliard block: 620 -> 140
+//   us; 1,089 rows in 2D, degree 16: 82 -> 25 us.
 // Rows are stored in slices of 32 (one warp), column-major within a slice and padded to its
 // longest row, so that every load of columns and values is one full line; rows next to each
 // other in Morton order have near-equal lengths.  With hanging nodes a row also holds the
