@@ -228,7 +228,11 @@ __device__ __forceinline__ double2 load2(const double* p, int64_t i, int64_t n) 
 __global__ void __launch_bounds__(CT, 1) cluster_kernel(double* V, int64_t ld, int k, Source src, int64_t n, double* __restrict__ sc,
                                                         double thr, double* host) {
     __shared__ double part[CW][257];   // sums of each warp: column j, then |w|^2
-    __shared__ double blk[2][257];     // of the block, per pass; read by the whole cluster
+    // of the block, per pass, read by the whole cluster: up to 256 columns, |w|^2 before the pass behind
+    // them (first pass) and after it in a slot of its own.  Nothing but a block barrier lies between the
+    // reads of the first two and the write of the last, so no column count may share a slot with it.
+    constexpr int AFTER = 257;
+    __shared__ double blk[2][AFTER + 1];
     __shared__ double fin[4][64], c[256], nrm[2][CW], bn[2];
     cg::cluster_group cl = cg::this_cluster();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -340,11 +344,11 @@ __global__ void __launch_bounds__(CT, 1) cluster_kernel(double* V, int64_t ld, i
             double s = 0.0;
 #pragma unroll
             for (int q = 0; q < CW; ++q) s += nrm[pass][q];
-            blk[pass][256] = s;
+            blk[pass][AFTER] = s;
         }
         cl.sync();
         if (warp == 0) {
-            double s = lane < CB ? *cl.map_shared_rank(&blk[pass][256], lane) : 0.0;
+            double s = lane < CB ? *cl.map_shared_rank(&blk[pass][AFTER], lane) : 0.0;
 #pragma unroll
             for (int o = CB / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             if (lane == 0) bn[1] = s;
