@@ -727,6 +727,9 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
         if ((st = dot_host(c, ws->dU, ws->dU, &du)) != CHNS_OK) return st;
         S.du_norm = std::sqrt(du);
     }
+    // a breakdown leaves the next vector's operator application in flight, on the caller's vectors and on
+    // the preconditioner's device description, which the next call may rewrite
+    if (result == CHNS_EBREAKDOWN) CHNS_CUDA(cudaStreamSynchronize(c.s));
     S.reason = result;
     if (stats) *stats = S;
     return result;

@@ -76,3 +76,21 @@ def test_newton_cycles_of_256_columns(chns, precision):
     U2, _ = chns.newton_step(gm, prm, chns.SolverOpts.make(pc_type=1, pc_degree=16, **kw), U0)
     assert U0.numel() <= 32768 and max(st.as_dict()["krylov_hist"]) > 2 * 256
     assert float((U1 - U2).norm()) <= 1e-9 * float(U2.norm())
+
+
+def test_breakdown_leaves_nothing_in_flight(chns):
+    """The call synchronises its stream, also where it gives up in the middle of an Arnoldi cycle with
+    the next operator application queued: velocities whose squares leave FP32 (not FP64) make the
+    operator's result not finite."""
+    gm, prm, U0 = problem(chns, 3, synth.uniform_leaves(3, 6), 6)
+    U0[:, :3] *= 1e25
+    opts = chns.SolverOpts.make(precision=1, pc_type=0, restart=30)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        out = torch.empty_like(U0)
+        torch.cuda.synchronize()
+        _, st = chns.newton_step(gm, prm, opts, U0, out, check=False)
+        idle = s.query()
+    torch.cuda.synchronize()
+    assert chns.STATUS[st.reason] == "CHNS_EBREAKDOWN" and st.jvp_calls == 2
+    assert idle
