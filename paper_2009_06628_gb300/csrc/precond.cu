@@ -768,7 +768,10 @@ __device__ void tail_cheb(const TailLevel& L, const float* in, float* out, float
 template <class TO>
 __global__ void __launch_bounds__(TAIL_THREADS) tail_kernel(const Tail* __restrict__ tp, TO* __restrict__ z, int NF, int f,
                                                             PrecondMean mean) {
-    __shared__ float sd[2][TAIL_ROWS];
+    union Scratch { float d[2][TAIL_ROWS]; double sum[TAIL_THREADS]; };   // directions; sums of the mean
+    static_assert(alignof(Scratch) >= alignof(double) && sizeof(Scratch) == sizeof(float) * 2 * TAIL_ROWS, "");
+    __shared__ Scratch sm;
+    float(*const sd)[TAIL_ROWS] = sm.d;
     chain_next<true>();
     chain_wait<true>();
     const Tail& T = *tp;
@@ -805,7 +808,7 @@ __global__ void __launch_bounds__(TAIL_THREADS) tail_kernel(const Tail* __restri
     }
     if (!mean.out) return;
     // four warps, one per scheduler, then one
-    double* sh = reinterpret_cast<double*>(sd);
+    double* const sh = sm.sum;
     sh[t0] = acc;
     __syncthreads();
     if (t0 < 128) {
