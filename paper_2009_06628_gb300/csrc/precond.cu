@@ -37,9 +37,21 @@ constexpr int MAX_DEG = 200;
 constexpr int CH_DEG = 8;
 constexpr int COARSE_DEG = 16;
 constexpr int TAIL_THREADS = 1024;
-// A level joins the one-block kernel when its matrix (8 B per entry) takes that SM about as long
-// as the launch that it saves: 40,960 entries are 328 KB, 2.5 us at 64 B per clock.
-constexpr int64_t TAIL_NNZ = 40960;
+constexpr int TAIL_ROWS = 2 * TAIL_THREADS;
+// Levels of the one-block kernel: those whose matrix its registers hold, from degree 5 on, and those
+// with so few entries that a step through L1 costs no more than a launched one.  A launched step is
+// 1.5 us at these sizes and one from registers 0.8; through L1 it is 1.5 at 2,601 entries and 6.4 at 38,025.
+//   Polynomial, degree 16, us per application, launched / here (block-Jacobi part included): 289 rows in 2D
+//   33 / 19, 1,089 rows 34 / 25, 729 rows in 3D 36 / 27; through L1: 2,681 rows in 2D with hanging points 34 / 88,
+//   4,225 rows 34 / 112, 1,049 rows in 3D with hanging points 50 / 96.
+//   V-cycle, degree 2, with all levels of up to 40,960 / 20,480 / 10,240 / 5,120 / 0 entries here: 66,049 rows in
+//   2D 122 / 89 / 89 / 81 / 81 us, 1,497 rows (hanging) 58 / 58 / 49 / 48 / 46, 365 rows 28 / 28 / 28 / 28 / 30,
+//   35,937 rows in 3D 66 / 66 / 60 / 60 / 60.
+//   Degree 4 on 1,089 rows: 17 launched, 17 from registers, 21 through L1; degree 2 from registers costs the
+//   V-cycle of that mesh 2 us.
+// The coarsest level of a V-cycle is always there (at most 300 rows, or level 1).
+constexpr int64_t TAIL_NNZ = 5120;
+constexpr int TAIL_DEG = 5;
 // Lanes per row: 4 where one thread per row would leave the chip short of loads in flight (a row
 // is a chain of 21 to 100 of them), 1 from 65,536 rows on.
 constexpr int64_t SPLIT_ROWS = 65536;
@@ -50,6 +62,7 @@ struct Sell {
     int64_t N = 0;
     int64_t ns = 0;            // slices
     int64_t nnz = 0;           // with padding
+    int wide = 0;              // longest row; known up to TAIL_ROWS rows
     int64_t* off = nullptr;    // ns + 1
     int32_t* col = nullptr;
 };
@@ -691,7 +704,6 @@ __device__ void tail_cheb_l(const TailLevel& L, const float* in, float* out) {
 // 1,089 rows of 9 (2D), degree 16: the kernel 34 -> 18 us (and a second one of 4.6 us, which stored the
 // result, went); 729 rows of 21 (3D): 17.2 -> 12.5 us; a V-cycle over 45,000 rows: 2 % of the
 // application.  Half the threads with twice the rows: 17.1, 13.7 us and 2 % slower.
-constexpr int TAIL_ROWS = 2 * TAIL_THREADS;
 template <int R, int W, int G, bool ADD>
 __device__ void tail_cheb_r(const TailLevel& L, const float* in, float* out, float (*sd)[TAIL_ROWS]) {
     const ChebCoef* cf = L.cf;
@@ -748,11 +760,12 @@ __device__ void tail_cheb_r(const TailLevel& L, const float* in, float* out, flo
         __syncthreads();
     }
 }
-// The register form where it fits and is long enough to pay for its loads; else from L1, eight lanes
-// per row where that leaves one round.
+// The register form where it fits and is long enough to pay for its loads (tail_regs tells the host); else
+// from L1, eight lanes per row where that leaves one round.  (With the form handed in by the host more
+// registers spill: the V-cycle of 1,049 rows takes 48 us instead of 46.)
 template <bool ADD>
 __device__ void tail_cheb(const TailLevel& L, const float* in, float* out, float (*sd)[TAIL_ROWS]) {
-    if (L.deg > 4 && L.S.N <= TAIL_ROWS) {
+    if (L.deg >= TAIL_DEG && L.S.N <= TAIL_ROWS) {
         int w = 0;
         for (int64_t s = threadIdx.x; s < L.S.ns; s += TAIL_THREADS)
             w = max(w, (int)((__ldg(L.S.off + s + 1) - __ldg(L.S.off + s)) >> 5));
@@ -964,6 +977,12 @@ cudaError_t sell_build(const Level& L, Sell& S, cudaStream_t s) {
         chns_count_launches(2);
         e = scan(width, T.ns, T.off, &T.nnz, s);
     }
+    if (e == cudaSuccess && m.N <= TAIL_ROWS) {
+        int32_t w[TAIL_ROWS / 32];
+        e = cudaMemcpyAsync(w, width, (size_t)T.ns * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) T.wide = *std::max_element(w, w + T.ns) / 32;
+    }
     if (e == cudaSuccess) e = alloc(&T.col, T.nnz);
     if (e == cudaSuccess) {
         sell_cols_kernel<EDGE, true><<<blocks_for(m.N * 32), 256, 0, s>>>(m, L.ip, L.inc, nullptr, T.off, T.col);
@@ -994,12 +1013,19 @@ void level_free(Level& L) {
 int level_degree(const PrecondWS* p, const PrecondSpec& spec, int l) {
     return spec.mg && l + 1 == (int)p->lv.size() ? COARSE_DEG : spec.degree;
 }
-// first level of the one-block kernel; with the polynomial alone, 0 when the mesh is small
+// whether tail_cheb takes the register form for a level
+bool tail_regs(const Sell& S, int deg) {
+    return deg >= TAIL_DEG && ((S.N <= TAIL_THREADS && S.wide <= 24) || (S.N <= TAIL_ROWS && S.wide <= 12));
+}
+// first level of the one-block kernel: 0 when the whole operator runs there, the number of levels when a
+// polynomial does not use it (a V-cycle always does)
 int first_tail(const PrecondWS* p, const PrecondSpec& spec) {
     const int nl = spec.mg ? (int)p->lv.size() : 1;
-    for (int l = 0; l < nl; ++l)
-        if (p->lv[(size_t)l].S.nnz <= TAIL_NNZ) return l;
-    return nl;
+    for (int l = 0; l < nl; ++l) {
+        const Sell& S = p->lv[(size_t)l].S;
+        if (S.nnz <= TAIL_NNZ || tail_regs(S, level_degree(p, spec, l))) return l;
+    }
+    return spec.mg ? nl - 1 : nl;
 }
 chns_status tail_describe(chns_mesh* m, const PrecondSpec& spec) {
     PrecondWS* p = m->pre;
