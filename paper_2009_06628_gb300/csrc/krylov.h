@@ -19,9 +19,11 @@ enum {
 
 namespace krylov {
 
-constexpr int T = 256;   // threads per block at most
+constexpr int T = 256;          // threads per block
+constexpr int COLUMNS = 256;    // at most
+constexpr int COUNTERS = 32;    // one per chunk of columns
 
-// sum over the block of K values per thread, to sh[0..K) of warp 0's lanes (T threads)
+// sum over the warp, in every lane (all 32 call it)
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -55,9 +57,9 @@ struct Source {
 // Gram-Schmidt of w (slot k of V, or formed there from src) against slots 0..k-1: coefficients,
 // norms and s_k in sc; host (pinned) gets the coefficients of both passes together in [0, k) and
 // |w|^2 in [SC_NA].  thr: re-orthogonalise when |w|^2 falls below thr times its old value (infinity:
-// always).  One launch for short vectors; else four, and two more per 32 columns beyond 32; returns
-// their number.
-// partials: 33 doubles for each of 16 blocks per SM; counter: zero.
+// always).  One launch for short vectors with few columns, else four, and two more per 32 columns beyond
+// 32 for long ones; returns their number.
+// partials: 33 doubles for each of 4 blocks per SM (of 8 SMs at least); counter: COUNTERS words, zero.
 int orthogonalise(double* V, int64_t ld, int k, const Source& src, int64_t n, double* sc, double thr, double* host, double* partials,
                   unsigned int* counter, cudaStream_t st);
 // u = sum_{j<k} y_j v_j

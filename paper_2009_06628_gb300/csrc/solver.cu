@@ -53,7 +53,7 @@ struct SolverWS {
     float* ce = nullptr;     // E element coefficients of the pressure Schur approximation
     double* part = nullptr;  // per-block partials of the Gram-Schmidt reductions
     double* mpart = nullptr; // and of the pressure mean
-    unsigned int* counter = nullptr;   // blocks that finished: Gram-Schmidt, pressure mean
+    unsigned int* counter = nullptr;   // blocks that finished: Gram-Schmidt (krylov::COUNTERS), pressure mean
     float* ch_psi2 = nullptr;  // psi''(phi~) at the nodes (Cahn-Hilliard block)
 };
 
@@ -131,10 +131,10 @@ chns_status ensure_ws(chns_mesh* m, int restart) {
     A((void**)&ws->Pinv64, nb * sizeof(double));
     A((void**)&ws->sc, MAXSC * sizeof(double));
     A((void**)&ws->ce, (size_t)m->dm.E * sizeof(float));
-    A((void**)&ws->part, (size_t)33 * 16 * chns_num_sms() * sizeof(double));   // 33 numbers of up to 16 blocks per SM
+    A((void**)&ws->part, (size_t)33 * 4 * std::max(chns_num_sms(), 8) * sizeof(double));   // 33 numbers of up to 4 blocks per SM
     A((void**)&ws->mpart, (size_t)(m->dm.N / 64 + 64) * sizeof(double));
-    A((void**)&ws->counter, 2 * sizeof(unsigned int));
-    if (e == cudaSuccess) e = cudaMemset(ws->counter, 0, 2 * sizeof(unsigned int));
+    A((void**)&ws->counter, (krylov::COUNTERS + 1) * sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMemset(ws->counter, 0, (krylov::COUNTERS + 1) * sizeof(unsigned int));
     A((void**)&ws->ch_psi2, (size_t)m->dm.N * sizeof(float));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&ws->hsc, MAXSC * sizeof(double));
     for (auto& ev : ws->ev)
@@ -454,7 +454,7 @@ extern "C" chns_status chns_newton_step(const chns_mesh* mc, const chns_params* 
     if (pin == 2) {
         pmn.nmass = m->d_nmass;
         pmn.partials = ws->mpart;
-        pmn.counter = ws->counter + 1;
+        pmn.counter = ws->counter + krylov::COUNTERS;
         pmn.out = ws->sc + SC_MEAN;
     }
     // Gram-Schmidt of Arnoldi step j on w = S J z (+ the rank-one term), with device-decided
@@ -819,7 +819,7 @@ extern "C" chns_status chns_step_adjoint(const chns_mesh* mc, const chns_params*
     // u^T lambda = 0 (GMRES on the singular J^T drifts along its null vector)
     const double inv_vol = 1.0 / m->volume;
     auto add_pmean_T = [&](const double* v, double* y) {
-        { field_wdot_kernel<<<nbw, 256, 0, c.s>>>(ws->Sd, v, NF, D, m->dm.N, m->d_partials, ws->counter + 1, ws->sc + SC_MISC + 1); chns_count_launches(1); }
+        { field_wdot_kernel<<<nbw, 256, 0, c.s>>>(ws->Sd, v, NF, D, m->dm.N, m->d_partials, ws->counter + krylov::COUNTERS, ws->sc + SC_MISC + 1); chns_count_launches(1); }
         { field_axpy_mass_kernel<<<c.g, 256, 0, c.s>>>(y, NF, D, m->dm.N, m->d_nmass, ws->sc + SC_MISC + 1, inv_vol); chns_count_launches(1); }
     };
     // b = P^T g: remove sum(g_p) * m / |Omega| from the pressure part (pin mode 2)

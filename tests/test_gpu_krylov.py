@@ -1,5 +1,5 @@
 """The Gram-Schmidt kernels at the edges of their ranges: Arnoldi cycles of up to 256 columns (the
-largest restart) on vectors that one cluster holds.  The adjoint solve with the FP64 block-Jacobi
+largest restart), and vector lengths of every split.  The adjoint solve with the FP64 block-Jacobi
 alone reports the residual of its Givens recursion, and the J^T w kernel gives the true one: they
 agree to 1 % (the solves stop at 1e-1 to 1e-6 of the right-hand side, where rounding is at
 1e-9, by the oracle's Jacobian in a host restatement of the same recursion)."""
@@ -94,3 +94,19 @@ def test_breakdown_leaves_nothing_in_flight(chns):
     torch.cuda.synchronize()
     assert chns.STATUS[st.reason] == "CHNS_EBREAKDOWN" and st.jvp_calls == 2
     assert idle
+
+
+@pytest.mark.parametrize("dim,lmin,level,band,n,its", [
+    (2, 4, 4, 0, 1445, 33), (2, 5, 5, 0, 5445, 70),                                # cluster, then 8 lanes per pair
+    (2, 5, 7, 0.02, 13605, 40), (2, 6, 7, 0.06, 34105, 70),                        # 4 lanes; 2, odd, past the cluster
+    (3, 4, 5, 0.01, 37518, 40), (3, 4, 5, 0.02, 46014, 70), (2, 7, 7, 0, 83205, 70),   # 2 lanes, 1 lane (even, odd)
+    (2, 9, 9, 0, 1315845, 40)])                                                    # a kernel per column count, odd, two launches
+def test_adjoint_over_the_splits(chns, dim, lmin, level, band, n, its):
+    """Column counts on both sides of 8, 32 and 64, vectors of each split of the work, odd and even."""
+    leaves = synth.uniform_leaves(dim, level) if lmin == level else \
+        synth.sphere_band_leaves(dim, lmin, level, [[0.5] * dim], [0.2 if n == 37518 else 0.25], band)
+    gm, prm, U0 = problem(chns, dim, leaves, level, pin_pressure=1)
+    assert U0.numel() == n
+    claim, true, norm, done = adjoint_claim(chns, gm, prm, U0, 256, its)
+    assert done == its
+    assert 0.0 < claim < norm and abs(true - claim) <= 0.01 * claim, (true, claim)
