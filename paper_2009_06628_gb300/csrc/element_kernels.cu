@@ -51,6 +51,27 @@ __device__ __forceinline__ void scatter_add(const DevMesh& m, T* __restrict__ ou
                                             const T r[Shape<D>::NF], unsigned skip0, int pair_rows, int pin) {
     constexpr int NF = Shape<D>::NF;
     const T w = parent_weight<T>(P.n);
+    if constexpr (SCAT == SCAT_PLAIN && sizeof(T) == 4) {
+        // a corner's parents differ: all of their rows are on the way before the first is written (the FP64
+        // kernels have no registers left for it)
+        unsigned skip[4];
+        T old[4][NF];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (j >= P.n) break;
+            skip[j] = j == 0 ? skip0 : replaced_rows<D>(m, parent(P, j), pin);
+#pragma unroll
+            for (int f = 0; f < NF; ++f) old[j][f] = out[(size_t)parent(P, j) * NF + f];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (j >= P.n) break;
+#pragma unroll
+            for (int f = 0; f < NF; ++f)
+                if (f > D || !((skip[j] >> f) & 1u)) out[(size_t)parent(P, j) * NF + f] = old[j][f] + w * r[f];
+        }
+        return;
+    }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         if (j >= P.n) break;
@@ -73,6 +94,25 @@ __device__ __forceinline__ void scatter_add(const DevMesh& m, T* __restrict__ ou
             else
                 atomicAdd(o + f, w * r[f]);
         }
+    }
+}
+
+// Plain adds of a warp's elements, LPE lanes each (SCAT_PLAIN; all lanes call it).  add(): this lane's rows;
+// hanging: whether its corner is.  The corners of an element that are nodes are distinct, so they add
+// together; a hanging corner's parents can be nodes of the element or another corner's parents, so
+// those add one after another, in a fixed order.  FP32 J x, us, with all corners in turn / so / with the
+// rows of scatter_add on the way together: 64^3 (8 colours) 320 / 263 / 173, a sphere on levels 3 to 6
+// 750 / 685 / 515; one thread per corner took 295 and 543.
+template <int LPE, class Add>
+__device__ __forceinline__ void plain_adds(int t, bool valid, bool hanging, Add add) {
+    if (valid && !hanging) add();
+    __syncwarp();
+    unsigned turns = __ballot_sync(0xffffffffu, valid && hanging);
+#pragma unroll
+    for (int o = LPE; o < 32; o <<= 1) turns |= turns >> o;
+    for (turns &= (1u << LPE) - 1u; turns; turns &= turns - 1u) {
+        if (valid && hanging && t == __ffs(turns) - 1) add();
+        __syncwarp();
     }
 }
 
@@ -213,13 +253,7 @@ elem_rj_kernel(DevMesh m, const __grid_constant__ Q1Params<S> prm, const typenam
             if (SCAT == SCAT_WARPAGG) {
                 scatter_add_warpagg<D, T>(m, out, P, rh, valid, wbuf[threadIdx.x >> 5], pin);
             } else if (SCAT == SCAT_PLAIN) {
-                // corners of one element can share a parent node (hanging corners): they add one
-                // after another, in a fixed order; elements of one colour share no node
-#pragma unroll 1
-                for (int a = 0; a < LPE; ++a) {
-                    if (valid && t == a) scatter_add<D, T, SCAT_PLAIN>(m, out, P, rh, skip0, 0, pin);
-                    __syncwarp();
-                }
+                plain_adds<LPE>(t, valid, P.n > 1, [&] { scatter_add<D, T, SCAT_PLAIN>(m, out, P, rh, skip0, 0, pin); });
             } else if (valid) {
                 scatter_add<D, T, SCAT>(m, out, P, rh, skip0, pair_rows, pin);
             }
@@ -337,32 +371,28 @@ elem_vjp_kernel(DevMesh m, const __grid_constant__ Q1Params<double> prm, double 
     {
         const Parents P = parents_of(m, ent);
         const double wt = parent_weight<double>(P.n);
-        // plain adds (colouring): the corners of an element add one after another (two
-        // corners can share a constraint parent); elements of one colour share no node
-#pragma unroll 1
-        for (int a = 0; a < (SCAT == SCAT_PLAIN ? NC : 1); ++a) {
-            if (valid && (SCAT != SCAT_PLAIN || t == a)) {
+        const auto add = [&] {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (j >= P.n) break;
-                    double* on = gn + (size_t)parent(P, j) * NF;
-                    double* oo = go ? go + (size_t)parent(P, j) * NF : nullptr;
-                    const double pst = (mask & (1u << j)) ? psb : 0.0;
+            for (int j = 0; j < 4; ++j) {
+                if (j >= P.n) break;
+                double* on = gn + (size_t)parent(P, j) * NF;
+                double* oo = go ? go + (size_t)parent(P, j) * NF : nullptr;
+                const double pst = (mask & (1u << j)) ? psb : 0.0;
 #pragma unroll
-                    for (int f = 0; f < NF; ++f) {
-                        const double vn = wt * (f == D + 1 ? rn[f] + pst : rn[f]);
-                        if (SCAT == SCAT_PLAIN) on[f] += vn;
-                        else atomicAdd(on + f, vn);
-                        if (oo) {
-                            const double vo = wt * (f == D + 1 ? ro[f] + pst : ro[f]);
-                            if (SCAT == SCAT_PLAIN) oo[f] += vo;
-                            else atomicAdd(oo + f, vo);
-                        }
+                for (int f = 0; f < NF; ++f) {
+                    const double vn = wt * (f == D + 1 ? rn[f] + pst : rn[f]);
+                    if (SCAT == SCAT_PLAIN) on[f] += vn;
+                    else atomicAdd(on + f, vn);
+                    if (oo) {
+                        const double vo = wt * (f == D + 1 ? ro[f] + pst : ro[f]);
+                        if (SCAT == SCAT_PLAIN) oo[f] += vo;
+                        else atomicAdd(oo + f, vo);
                     }
                 }
             }
-            if (SCAT == SCAT_PLAIN) __syncwarp();
-        }
+        };
+        if (SCAT == SCAT_PLAIN) plain_adds<NC>(t, valid, P.n > 1, add);
+        else if (valid) add();
     }
     if (gCn) {
         // each Gauss point thread holds its share of d/dCn
