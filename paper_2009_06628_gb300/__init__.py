@@ -143,10 +143,15 @@ def _check(code):
 
 
 # The smallest calls are bound by the host (J x on 32^2 in FP64: 17.6 to 12.9 us of host time per call, for
-# 14 us on the device): addresses go to ctypes as integers, and the
-# stream's without a torch.cuda.Stream object around it.
+# 14 us on the device): addresses go to ctypes as integers, and the stream's without a torch.cuda.Stream
+# object around it, where torch offers that (the name is not part of its public interface).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream():
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _ptr(t, dtype=torch.float64):
