@@ -241,7 +241,7 @@ elem_rj_kernel(DevMesh m, const __grid_constant__ Q1Params<S> prm, const typenam
         }
         S r[NF];
 #pragma unroll
-        for (int f = 0; f < NF; ++f) r[f] = mul2(L.vol, q1_vgradT<D, false>(prm.f, prm.fr, F0[f], F1[f], (const S*)nullptr));
+        for (int f = 0; f < NF; ++f) r[f] = mul2(L.vol, q1_vgradT<D, false>(prm.fc, prm.fcr, F0[f], F1[f], (const S*)nullptr));
         chain_wait<true>();
 #pragma unroll
         for (int h = 0; h < NP; ++h) {
@@ -326,7 +326,7 @@ elem_vjp_kernel(DevMesh m, const __grid_constant__ Q1Params<double> prm, double 
         for (int f = 0; f < NF; ++f) {
             double t;
             q1_vgrad<D, false>(P.n == 1 ? sw[f] : wt * sw[f], t, F1[f], (double*)nullptr);
-            F0[f] = prm.f * t;
+            F0[f] = prm.fc * t;
         }
     }
     PwIn<D, double> B;

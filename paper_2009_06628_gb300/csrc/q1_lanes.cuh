@@ -207,6 +207,7 @@ template <class S>
 struct Q1Params {
     PwConst<S> c;
     S f, fr, inv_f;          // f, f r, 1/f
+    S fc, fcr;               // f and f r of the test contraction, which rounds against f: f fc = f^2
     S sp;                    // f/We
     S sd;                    // scale of time differences: c_+^d/dt
     PwLevel<S> lev[Q1_LEVELS];
@@ -224,14 +225,21 @@ Q1Params<S> q1_params(const PhysConst& pc, double span, int max_level) {
     p.c.td = splat<S>(2.0 * pc.inv_dt);
     p.c.c0 = splat<S>(pc.four_over_dt2);
     p.c.inv_We = splat<S>(pc.inv_We);
-    p.c.gk = splat<S>(4.0 * Q1_CP * Q1_CP / (f * f));
+    // s, s^2 and gk from powers of c_+, not from the rounded f: a constant's rounding is an error of every
+    // entry alike (s^2 of f/c_+ in 2D: 2.1e-16), and so is that of f, which enters twice (2D FP32: -8.1e-8 with
+    // f in both places, 1.5e-8 with fc)
+    const double c = D == 2 ? Q1_CP : Q1_CP * Q1_CP;
+    p.c.gk = splat<S>(16.0 / (c * c));
+    const double fc = sizeof(typename Scalar<S>::type) == 4 ? f * f / (double)(float)f : f;
     p.f = splat<S>(f);
     p.fr = splat<S>(f * Q1_R);
+    p.fc = splat<S>(fc);
+    p.fcr = splat<S>(fc * Q1_R);
     p.inv_f = splat<S>(1.0 / f);
     p.sp = splat<S>(f * pc.inv_We);
     p.sd = splat<S>(cd * pc.inv_dt);
     for (int l = 0; l < Q1_LEVELS; ++l) {
-        const double h = ldexp(span, -(l <= max_level ? l : max_level)), s = f / (h * Q1_CP), kap = s * s;
+        const double h = ldexp(span, -(l <= max_level ? l : max_level)), s = 0.5 * c / h, kap = 0.25 * (c * c) / (h * h);
         const double g = 4.0 / (h * h);
         PwLevel<S>& L = p.lev[l];
         L.s = splat<S>(s);
