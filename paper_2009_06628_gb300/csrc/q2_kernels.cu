@@ -86,10 +86,22 @@ struct Tri {
     __device__ __forceinline__ S der(const Line<S>& l) const { return fma3(l.D[2], q, fma3(l.D[1], p, mul2(l.D[0], o))); }
     __device__ __forceinline__ S val(const Line<S>& l, S c) const { return fma3(l.L[2], q, fma3(l.L[1], p, fma3(l.L[0], o, c))); }
     __device__ __forceinline__ S der(const Line<S>& l, S c) const { return fma3(l.D[2], q, fma3(l.D[1], p, fma3(l.D[0], o, c))); }
+};
+// The same from the differences to the own value, for values and derivatives of nodal data together (no more
+// operations: L sums to 1 and D to 0 over a line).  A derivative as a sum of products rounds at the size of
+// the data, which in the phases is 1 where the derivative is 0; so it rounds at the size of the variation.
+//   Against 64 bits, 2D 32^2: solenoidality row of the residual 6.1e-15 -> 3.4e-15, potential row 7.9e-15 ->
+//   5.5e-15, all rows 9.6e-16 -> 8.1e-16, FP32 J x 1.0e-7 -> 8.4e-8.  (8^3 and 16^3 FP64 J x and residual: 3 %
+//   less time.)
+template <class S>
+struct Dif {
+    S o, p, q;
+    __device__ __forceinline__ Dif(S u, const Line<S>& l) : o(u), p(sub2(shfl(u, l.n1), u)), q(sub2(shfl(u, l.n2), u)) {}
+    __device__ __forceinline__ S val(const Line<S>& l) const { return fma3(l.L[2], q, fma3(l.L[1], p, o)); }
+    __device__ __forceinline__ S der(const Line<S>& l) const { return fma3(l.D[2], q, mul2(l.D[1], p)); }
     // u_0 - 2 u_1 + u_2, the second derivative at every point of the line
     __device__ __forceinline__ S sec(const Line<S>& l) const {
-        const S mid = l.d == 1 ? o : (l.d == 0 ? p : q);
-        return fma3(splat<S>(-3.0), mid, add2(add2(o, p), q));
+        return fma3(splat<S>(l.d == 1 ? 1.0 : -2.0), l.d == 0 ? p : q, l.d == 0 ? q : p);
     }
 };
 // transpose of sec, with the weights: node a collects (1, -2, 1)_a times the line's weighted sum
@@ -103,9 +115,11 @@ __device__ __forceinline__ S sec_t(S u, const Line<S>& l) {
 // value, D_k gradient; HS: mixed (h) and pure (hd) second derivatives; LP: Laplacian
 template <int D, bool HS, bool LP, class S>
 __device__ __forceinline__ void q2_vgrad(S u, const Line<S> l[D], S& val, S g[D], S* h, S* hd, S* lap) {
-    const Tri<S> t(u, l[0]);
+    using Along = std::conditional_t<HS, Dif<S>, Tri<S>>;   // Tri: the value alone
+    const Dif<S> t(u, l[0]);
     const S A = t.val(l[0]), B = t.der(l[0]);
-    const Tri<S> ta(A, l[1]), tb(B, l[1]);
+    const Dif<S> ta(A, l[1]);
+    const Along tb(B, l[1]);
     const S AA = ta.val(l[1]), AB = ta.der(l[1]), BA = tb.val(l[1]);
     S EA, AE;
     if (HS || LP) {
@@ -123,7 +137,8 @@ __device__ __forceinline__ void q2_vgrad(S u, const Line<S> l[D], S& val, S g[D]
         }
         if (LP) *lap = add2(EA, AE);
     } else {
-        const Tri<S> taa(AA, l[2]), tab(AB, l[2]), tba(BA, l[2]);
+        const Dif<S> taa(AA, l[2]);
+        const Along tab(AB, l[2]), tba(BA, l[2]);
         val = taa.val(l[2]);
         g[2] = taa.der(l[2]);
         g[1] = tab.val(l[2]);
@@ -194,10 +209,14 @@ __device__ __forceinline__ void q2_vder(S u, const Line<S> l[D], S& val, S& g) {
     val = u;
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-        const Tri<S> t(val, l[k]);
         if (k > K) g = Tri<S>(g, l[k]).val(l[k]);
-        if (k == K) g = t.der(l[k]);
-        val = t.val(l[k]);
+        if (k == K) {
+            const Dif<S> t(val, l[k]);
+            g = t.der(l[k]);
+            val = t.val(l[k]);
+        } else {
+            val = Tri<S>(val, l[k]).val(l[k]);
+        }
     }
 }
 template <int D, int K, class S>
