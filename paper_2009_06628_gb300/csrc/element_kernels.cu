@@ -14,12 +14,12 @@
 // What bounds them: FP64, the FP64 pipe (2 lanes per SM and clock), so operations per Gauss
 // point are the whole cost: lane-exchange interpolation and the regrouped pointwise map
 // (point_physics.cuh) brought them, on 64^3 elements, from 925 / 1471 / 1753 to about 365 /
-// 580 / 720 for the residual, J x and J^T w: 3.08 / 4.90 / 5.85 ms -> 1.37 / 2.23 / 2.56 ms
+// 580 / 720 for the residual, J x and J^T w: 3.08 / 4.90 / 5.85 ms -> 1.39 / 2.25 / 2.60 ms
 // (one thread per Gauss point with shared-memory corners and dual numbers before).
-// FP32 J x: 543 instead of 1696 instructions per Gauss point (packed pairs); 64^3 130 -> 72 us,
-// 128^3 997 -> 484 us per call.  It now waits for its gathers: 160 registers leave 12 warps per
+// FP32 J x: 543 instead of 1696 instructions per Gauss point (packed pairs); 64^3 135 -> 69 us,
+// 128^3 997 -> 491 us per call.  It now waits for its gathers: 168 registers leave 12 warps per
 // SM (ncu: half of the stall cycles on global loads, FMA pipe 40 %, shuffle/load unit 52 %).
-// 2 or 4 resident blocks instead of 3: 128^3 571 / 716 us.
+// 2 or 4 resident blocks instead of 3: 128^3 571 / 716 us (484 at the time).
 #include <cuda_runtime.h>
 
 #include <type_traits>

@@ -10,7 +10,7 @@
 // kernel gathers, reduces and updates: half the chain, no atomics, a fixed summation order.
 //   64^3 (274,625 rows), degree 16: a whole preconditioner application 313 -> 125 us (15 of them the
 //   block-Jacobi part); 45,000 rows with hanging points, V-cycle and Cahn-Hilliard block: 620 -> 140
-//   us; 1,089 rows in 2D, degree 16: 82 -> 25 us.
+//   us; 1,089 rows in 2D, degree 16: 90 -> 25 us.
 // Rows are stored in slices of 32 (one warp), column-major within a slice and padded to its
 // longest row, so that every load of columns and values is one full line; rows next to each
 // other in Morton order have near-equal lengths.  With hanging nodes a row also holds the
@@ -417,7 +417,7 @@ __device__ __forceinline__ int64_t my_row(int64_t N, bool& store) {
 // diagonal, coefficients), and waits there.  Every thread waits before it touches a vector, so a link
 // that is done implies that all earlier ones are.  Vectors are then read with plain loads: the
 // read-only path asks that nobody writes them meanwhile.  V-cycle and Cahn-Hilliard block on 45,000
-// rows: 163 -> 139 us.  Larger grids fill the chip, and a successor that waits would take its place.
+// rows: 163 -> 140 us.  Larger grids fill the chip, and a successor that waits would take its place.
 template <int LPR> constexpr bool LINK = LPR != 1;
 template <bool ON> __device__ __forceinline__ float vec(const float* x) { return ON ? *x : __ldg(x); }
 // A row of this lane group, its first PRE entries per lane already loaded

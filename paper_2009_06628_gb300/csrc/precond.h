@@ -43,7 +43,8 @@ struct PrecondMean {
     double* out = nullptr;
 };
 // Writes the pressure (schur) and phi, mu (ch) rows of z from the inputs.  Replayed from a CUDA
-// graph per (z, mean, spec).
+// graph per (z, mean, spec), four of which are kept; precond_prepare with another degree or kind of
+// pressure approximation drops them (there is one description of the one-block levels per mesh).
 chns_status precond_apply(chns_mesh* m, const PrecondSpec& spec, float* z, const PrecondMean& mean, cudaStream_t s);
 chns_status precond_apply(chns_mesh* m, const PrecondSpec& spec, double* z, const PrecondMean& mean, cudaStream_t s);
 // Captured graphs hold the callers' vectors: drop them when those are freed.

@@ -10,8 +10,8 @@
 // evaluation as much again.  The test contraction runs the transposes with the quadrature weights
 // in their coefficients.  Unlike Q1, the pure second derivatives do not vanish: the strong
 // residuals take the full Hessian of phi and the Laplacians of v and mu (pw_*<..., Q2 = true>).
-//   32^3 elements, FP32 J x: 303 -> 100 us; FP64 J x 10.2 -> 2.15 ms, residual 7.8 -> 1.33 ms,
-//   J^T w 11.2 -> 2.37 ms.
+//   32^3 elements, FP32 J x: 303 -> 94 us; FP64 J x 10.2 -> 2.04 ms, residual 7.8 -> 1.26 ms,
+//   J^T w 11.2 -> 2.31 ms.
 // Bound: FP64 pipe (FP64), shuffles and FMA issue in equal parts (FP32).
 #include <cuda_runtime.h>
 
